@@ -182,6 +182,43 @@ __device__ __forceinline__ void edge_grad(bool plm, bool right, const R *w, R &p
   }
 }
 
+// Transposed angular coefficients of bin n in a column (donor cell): what
+// divA of the bin itself and of its neighbours take from I_n.  With c_s the
+// prefactor of the flux out of n through side s, divA_n = sum_s c_s
+// I_up / dOmega_n, and the neighbour m across s sees -c_s I_up / dOmega_m (its
+// own table entry for the side):
+//   at_self = sum over sides with n upwind of c_s / dOmega_n,
+//   at_nb[s] = -c_s / dOmega_m where n is upwind, else 0.
+template <typename R, typename Col>
+__device__ __forceinline__ void side_transposed(const StageArgs &a, const Col &cg, int col, int n, bool act,
+                                                R &at_self, R (&at_nb)[kMaxSlots], int (&nb_m)[kMaxSlots]) {
+  at_self = R(0);
+  const bool tab = a.side_P != nullptr;
+  const unsigned up = tab && act ? a.side_up[(size_t)col * a.nap + n] : 0u;
+#pragma unroll
+  for (int s = 0; s < kMaxSlots; ++s) {
+    const int m = act ? a.nbr_t[s * a.nap + n] : 0;
+    at_nb[s] = R(0);
+    nb_m[s] = m;
+    if (!act || m == n) continue;
+    if (tab) {
+      if (!((up >> s) & 1u)) continue;
+      const R *row = (const R *)a.side_P + (size_t)col * kSideRows * a.nap;
+      at_self += row[s * a.nap + n];
+      at_nb[s] = row[a.rslot_t[s * a.nap + n] * a.nap + m];
+    } else {
+      const int e = a.slot_edge[6 * n + s];
+      const bool isp = a.edge_pq[2 * e] == n;
+      bool upp;
+      R c = side_prefactor<R>(cg, a.edge_geo + 8 * e, upp);
+      if (upp != isp) continue;
+      if (!isp) c = -c;
+      at_self += per_solid_angle(c, a.dOmega, a.rdO, n);
+      at_nb[s] = per_solid_angle(-c, a.dOmega, a.rdO, m);
+    }
+  }
+}
+
 // Transposed transport of one stage (gather form, one thread per target bin).
 // PPM: the spatial reconstruction is PPM (each face state depends on the five
 // cells around its upwind cell) instead of DC / PLM (three cells).
@@ -276,18 +313,7 @@ __global__ void __launch_bounds__(MAXT, sizeof(R) == 8 ? 1 : 1280 / MAXT) k_tran
   R ap_P[NE];
   int ap_e[NE], ap_p[NE], ap_q[NE], ap_u[NE], ap_d[NE], ap_b[NE];
   auto edge_P = [&](int e, bool &upp) -> R {
-      const double *eg = a.edge_geo + 8 * e;
-      const R x = (R)eg[0], yv = (R)eg[1], z = (R)eg[2], len = (R)eg[6];
-      const R pr[10] = {R(1), x, yv, z, x * x, x * yv, x * z, yv * yv, yv * z, z * z};
-      R q0 = R(0), q1 = R(0), q2 = R(0);
-      for (int p = 0; p < 10; ++p) {
-        q0 += cg.K[0][p] * pr[p];
-        q1 += cg.K[1][p] * pr[p];
-        q2 += cg.K[2][p] * pr[p];
-      }
-      const R sp = -((R)eg[3] * q0 + (R)eg[4] * q1 + (R)eg[5] * q2);
-      upp = sp >= R(0);                       // upwind: p (ties to p, as the forward)
-      return len * sp * (cg.M[0][0] + cg.M[0][1] * x + cg.M[0][2] * yv + cg.M[0][3] * z);
+    return side_prefactor<R>(cg, a.edge_geo + 8 * e, upp);     // upwind: p (ties to p, as the forward)
   };
   // MAPR (AM): every side's prefactor and upwind side for this column
   __shared__ R amP[AM ? 3 * kMaxBinsStep : 1];
@@ -337,42 +363,7 @@ __global__ void __launch_bounds__(MAXT, sizeof(R) == 8 ? 1 : 1280 / MAXT) k_tran
   // angular: transposed coefficients
   R at_self = R(0), at_nb[kMaxSlots];
   int nb_m[kMaxSlots];
-  if (ANG && !AP && !AM) {
-    R self = R(0);
-    for (int s = 0; s < kMaxSlots; ++s) {
-      at_nb[s] = R(0);
-      nb_m[s] = nb_self;
-      int m = act ? a.slot_nbr[6 * n + s] : -1;
-      if (m < 0) continue;
-      nb_m[s] = m;
-      int e = a.slot_edge[6 * n + s];
-      const double *eg = a.edge_geo + 8 * e;
-      R x = (R)eg[0], yv = (R)eg[1], z = (R)eg[2], v0 = (R)eg[3], v1 = (R)eg[4], v2 = (R)eg[5], len = (R)eg[6];
-      R pr[10] = {R(1), x, yv, z, x * x, x * yv, x * z, yv * yv, yv * z, z * z};
-      R q0 = R(0), q1 = R(0), q2 = R(0);
-      for (int p = 0; p < 10; ++p) {
-        q0 += cg.K[0][p] * pr[p];
-        q1 += cg.K[1][p] * pr[p];
-        q2 += cg.K[2][p] * pr[p];
-      }
-      R sp = -(v0 * q0 + v1 * q1 + v2 * q2);
-      R n0e = cg.M[0][0] + cg.M[0][1] * x + cg.M[0][2] * yv + cg.M[0][3] * z;
-      R P = len * sp * n0e;
-      R PL = sp >= R(0) ? P : R(0), PR = sp >= R(0) ? R(0) : P;
-      R dOm_m = (R)a.dOmega[m];
-      // forward: divA_n gets (n == p ? PL : -PR) / dOm_n from I_n and
-      // (n == p ? PR : -PL) / dOm_n from I_m; the transpose gathers what
-      // divA_m takes from I_n
-      if (a.edge_pq[2 * e] == n) {
-        self += PL / dOm;
-        at_nb[s] = -PL / dOm_m;
-      } else {
-        self -= PR / dOm;
-        at_nb[s] = PR / dOm_m;
-      }
-    }
-    at_self = act ? self : R(0);
-  }
+  if (ANG && !AP && !AM) side_transposed<R>(a, cg, col, n, act, at_self, at_nb, nb_m);
   // neighbour addressing along x1 / x2 (periodic wrap, outflow clamp; polar
   // positions are handled separately).  A polar position further from the
   // pole than the line is long mirrors to no row (the index returned is then

@@ -21,6 +21,9 @@ void free_angles(rad::DevAngles &d) {
   cudaFree(d.dOmega);
   cudaFree(d.slot_nbr);
   cudaFree(d.slot_edge);
+  cudaFree(d.nbr_t);
+  cudaFree(d.rslot_t);
+  cudaFree(d.rdO);
   cudaFree(d.perm);
   cudaFree(d.edge_geo);
   cudaFree(d.edge_pq);
@@ -121,6 +124,18 @@ static int install_angles(rad_ctx *ctx, AngleGrid &g, int *n_ang_out, int *n_ang
   std::vector<int> snb(6 * g.n_ap, -1), sed(6 * g.n_ap, -1), perm(g.n_ap, 0);
   std::vector<int> lbh(g.line_behind.empty() ? 0 : rad::kMaxBehind * g.n_ap, -1);   // padded bins: none
   for (size_t q = 0; q < g.line_behind.size(); ++q) lbh[q] = g.line_behind[q];
+  std::vector<int> nbt(6 * g.n_ap, 0);
+  std::vector<unsigned char> rsl(6 * g.n_ap, 0);
+  std::vector<double> rdo(g.n_ap, 0.0);
+  for (int n = 0; n < g.n_ang; ++n) {
+    rdo[n] = 1.0 / g.dOmega[n];
+    for (int s = 0; s < 6; ++s) {
+      const int m = g.nbr[6 * n + s];
+      nbt[s * g.n_ap + n] = m >= 0 ? m : n;
+      for (int r = 0; m >= 0 && r < 6; ++r)
+        if (g.slot_edge[6 * m + r] == g.slot_edge[6 * n + s]) rsl[s * g.n_ap + n] = (unsigned char)r;
+    }
+  }
   // minimum-angle plane tables, padded to n_ap bins (padding: no neighbours)
   const bool mapr = !g.mapr_nb.empty();
   std::vector<int> mnb(mapr ? 6 * g.n_ap : 0, -1);
@@ -152,6 +167,9 @@ static int install_angles(rad_ctx *ctx, AngleGrid &g, int *n_ang_out, int *n_ang
       (ce = upload(&ctx->dang.dOmega, dOm, ctx->stream)) != cudaSuccess ||
       (ce = upload(&ctx->dang.slot_nbr, snb, ctx->stream)) != cudaSuccess ||
       (ce = upload(&ctx->dang.slot_edge, sed, ctx->stream)) != cudaSuccess ||
+      (ce = upload(&ctx->dang.nbr_t, nbt, ctx->stream)) != cudaSuccess ||
+      (ce = upload(&ctx->dang.rslot_t, rsl, ctx->stream)) != cudaSuccess ||
+      (ce = upload(&ctx->dang.rdO, rdo, ctx->stream)) != cudaSuccess ||
       (ce = upload(&ctx->dang.perm, perm, ctx->stream)) != cudaSuccess ||
       (ce = upload(&ctx->dang.edge_geo, egeo, ctx->stream)) != cudaSuccess ||
       (ce = upload(&ctx->dang.edge_pq, g.edge_pq, ctx->stream)) != cudaSuccess ||
@@ -392,6 +410,7 @@ int rad_step(rad_ctx *ctx, void *I, const rad_gas *gas, double dt, const rad_opt
   int st = rad::check_step_args(ctx, I, gas, dt, o);
   if (st != RAD_OK) return st;
   if ((st = ensure_scratch(ctx, o)) != RAD_OK) return st;
+  rad::ensure_side_table(ctx, o->precision);
   ctx->stage1_prec = -1;    // the scratch no longer holds a rad_step_stage stage-1 result
   std::string err;
   if (ctx->n_groups > 0)
@@ -416,6 +435,7 @@ int rad_step_stage(rad_ctx *ctx, int stage, void *I, const rad_gas *gas, double 
   const size_t esz = o->precision == RAD_F32 ? 4 : 8;
   if (stage == 1) {
     if ((st = ensure_scratch(ctx, o)) != RAD_OK) return st;
+    rad::ensure_side_table(ctx, o->precision);
     ctx->stage1_prec = o->precision;
   } else if (ctx->stage1_prec != o->precision || ctx->scratch_I_bytes < ncell * ctx->ang.n_ap * esz ||
              ctx->scratch_T_count < ncell) {
@@ -509,6 +529,7 @@ int rad_step_adjoint(rad_ctx *ctx, const void *I_n, const rad_gas *gas, double d
   if (!(dt > 0.0)) return fail(ctx, RAD_EINVAL, "dt must be > 0");
   if (ctx->ang.n_ang > rad::kMaxBinsStep)
     return fail(ctx, RAD_EUNSUPPORTED, "rad_step_adjoint supports up to 812 bins (geodesic level 9)");
+  rad::ensure_side_table(ctx, o->precision);
   std::string err;
   st = rad::launch_adjoint(ctx, I_n, gas, dt, o, lam_np1, lam_n, lamT_np1, lamT_n, g_aa, g_as, g_eta, err);
   return st == RAD_OK ? st : fail(ctx, st, err);

@@ -338,6 +338,12 @@ void free_geometry(DevGeom &g) {
   cudaFree(g.f2F);
   cudaFree(g.f3F);
   cudaFree(g.xf_dev);
+  for (int p = 0; p < 2; ++p) {
+    cudaFree(g.side_P[p]);
+    cudaFree(g.side_up[p]);
+    g.side_P[p] = nullptr;
+    g.side_up[p] = nullptr;
+  }
   g.cols = nullptr;
   g.f1 = g.f2 = g.f3 = nullptr;
   g.colsF = nullptr;

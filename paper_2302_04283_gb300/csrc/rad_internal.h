@@ -15,6 +15,7 @@ constexpr double kPi = 3.14159265358979323846;
 constexpr int kMaxBinsStep = 812;        // rad_step: one CTA of <= 512 threads holds all bins of a cell
                                          // (812 = geodesic level 9)
 constexpr int kMaxSlots = 6;             // neighbours of a geodesic cell
+constexpr int kSideRows = kMaxSlots + 1; // rows of the side table per column
 constexpr int kMaxBehind = 4;            // sides whose line reconstruction reads a lat/long cell as
                                          // the cell behind (one per line direction)
 
@@ -92,6 +93,9 @@ struct DevAngles {
   double *dOmega = nullptr;    // [n_ap]
   int *slot_nbr = nullptr;     // [n_ap][6]
   int *slot_edge = nullptr;    // [n_ap][6]
+  int *nbr_t = nullptr;        // [6][n_ap] neighbours, slot-major; the bin itself where there is none
+  unsigned char *rslot_t = nullptr;   // [6][n_ap] slot of the same side in that neighbour's list
+  double *rdO = nullptr;       // [n_ap] 1 / dOmega (0 in padding)
   int *perm = nullptr;         // [n_ap]
   double *edge_geo = nullptr;  // [n_edge][8]: mid xyz, nrm xyz, len, p-index
   int *edge_pq = nullptr;      // [n_edge][2]
@@ -116,6 +120,14 @@ struct DevGeom {
   ColGeoF *colsF = nullptr;    // float copies of the above
   FaceGeoF *f1F = nullptr, *f2F = nullptr, *f3F = nullptr;
   double *xf_dev = nullptr;    // packed face coordinates
+  // angular-flux prefactors of every column (curved metrics; index 0 FP64, 1
+  // FP32; built by the first step of that precision, see ensure_side_table):
+  // side_P [col][7][n_ap], rows 0..5 = +-len (V . nu) n_0 / dOmega of the bin's
+  // sides, oriented out of the bin (0 where there is no side), row 6 the sum
+  // of those whose upwind cell is the bin itself; side_up [col][n_ap], bit s
+  // set where the bin is upwind of its side s
+  void *side_P[2] = {nullptr, nullptr};
+  unsigned char *side_up[2] = {nullptr, nullptr};
 };
 
 }  // namespace rad
@@ -192,6 +204,11 @@ int launch_halo_pack(rad_ctx *ctx, const void *I, int precision, int dim, int si
 constexpr int kHaloLayers = 3;   // the widest stencil (PPM) reaches three cells
 int launch_cfl(rad_ctx *ctx, double cfl, double *dt_out, std::string &err);
 cudaError_t launch_wait_selftest(rad_ctx *ctx, double seconds);
+
+// sides.cu: build the side table of a precision if the metric has angular
+// fluxes and the table is worth its memory; without one the kernels compute
+// the prefactors themselves (the same values)
+void ensure_side_table(rad_ctx *ctx, int precision);
 
 // moments.cu
 int launch_moments(rad_ctx *ctx, const void *I, int precision, int frame, int method,

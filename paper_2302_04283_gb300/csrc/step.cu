@@ -164,6 +164,11 @@ StageArgs make_stage_args(rad_ctx *ctx, const rad_gas *gas, double dt, const rad
   a.perm = ctx->dang.perm;
   a.slot_nbr = ctx->dang.slot_nbr;
   a.slot_edge = ctx->dang.slot_edge;
+  a.nbr_t = ctx->dang.nbr_t;
+  a.rslot_t = ctx->dang.rslot_t;
+  a.rdO = ctx->dang.rdO;
+  a.side_P = G.side_P[o->precision == RAD_F32];
+  a.side_up = G.side_up[o->precision == RAD_F32];
   a.edge_pq = ctx->dang.edge_pq;
   a.edge_line = ctx->dang.edge_line;
   a.line_behind = ctx->dang.line_behind;

@@ -44,6 +44,7 @@
 #include <string>
 
 #include "rad_internal.h"
+#include "sides.cuh"
 
 namespace rad {
 
@@ -72,6 +73,11 @@ struct StageArgs {
   const void *f1, *f2, *f3;
   const double *dir, *dOmega, *edge_geo;
   const int *perm, *slot_nbr, *slot_edge, *edge_pq;
+  const int *nbr_t;        // [6][nap] neighbours, slot-major (own bin where none)
+  const unsigned char *rslot_t;   // [6][nap] slot of the side in the neighbour's list
+  const double *rdO;       // 1 / dOmega
+  const void *side_P;      // side table of this precision (null: formed by the kernels)
+  const unsigned char *side_up;
   const int *edge_line;    // latitude-longitude grids: cell behind p, cell beyond q of each side
   const int *line_behind;  // latitude-longitude grids: per bin, the sides it is the cell behind of (adjoint)
   int n_edge;              // sides of the angle grid
@@ -904,66 +910,74 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
   R xu[2][kMaxSlots][2];      // MAPR: gnomonic coordinates of each side's midpoint in its upwind cell's plane
   int nb_m[2][kMaxSlots];
   if (ANG) {
-    // unrolled in FP32 so that the coefficients stay in registers; the FP64
-    // kernels keep them in local memory (they are bound by the FP64 pipe)
-#pragma unroll(sizeof(R) == 4 ? 2 : 1)
-    for (int e = 0; e < 2; ++e) {
-      const int n = b0 + e;
-      const bool ac = n < a.nang;
-      R self = R(0);
+    // the prefactors (per solid angle) of the flux out of the bin through each
+    // side, from the side table (one coalesced row per slot) or, where there
+    // is none, formed here.  Unrolled in FP32 so that the coefficients stay
+    // in registers; the FP64 kernels keep them in local memory (they are
+    // bound by the FP64 pipe)
+    const bool tab = a.side_P != nullptr;
+    const int bs = inpair ? b0 : 0;
+    const R *trow = (const R *)a.side_P + (size_t)col * kSideRows * nap + bs;
+    unsigned upm[2] = {0u, 0u};
+    if (tab) {
+      const uchar2 m2 = *(const uchar2 *)(a.side_up + (size_t)col * nap + bs);
+      upm[0] = m2.x;
+      upm[1] = m2.y;
+    }
+#pragma unroll(sizeof(R) == 4 ? kMaxSlots : 1)
+    for (int s = 0; s < kMaxSlots; ++s) {
+      const V tv = tab ? __ldg((const V *)(trow + s * nap)) : P::mk(R(0), R(0));
+      const int2 mv = *(const int2 *)(a.nbr_t + s * nap + bs);
 #pragma unroll
-      for (int s = 0; s < kMaxSlots; ++s) {
-        a_nb[e][s] = R(0);
-        nb_m[e][s] = ac ? n : 0;
-        xu[e][s][0] = xu[e][s][1] = R(0);
-        int m = ac ? a.slot_nbr[6 * n + s] : -1;
-        if (m < 0) continue;
+      for (int e = 0; e < 2; ++e) {
+        const int n = b0 + e;
+        const bool ac = n < a.nang;
+        const int m = ac ? (e ? mv.y : mv.x) : 0;
         nb_m[e][s] = m;
-        int ed = a.slot_edge[6 * n + s];
-        const double *eg = a.edge_geo + 8 * ed;
-        R x = (R)eg[0], y = (R)eg[1], z = (R)eg[2], v0 = (R)eg[3], v1 = (R)eg[4], v2 = (R)eg[5], len = (R)eg[6];
-        R pr[10] = {R(1), x, y, z, x * x, x * y, x * z, y * y, y * z, z * z};
-        R q0 = R(0), q1 = R(0), q2 = R(0);
-#pragma unroll
-        for (int p = 0; p < 10; ++p) {
-          q0 += cg.K[0][p] * pr[p];
-          q1 += cg.K[1][p] * pr[p];
-          q2 += cg.K[2][p] * pr[p];
+        a_nb[e][s] = R(0);
+        xu[e][s][0] = xu[e][s][1] = R(0);
+        if (!ac || m == n) continue;
+        R cs = e ? tv.y : tv.x;
+        bool upn = (upm[e] >> s) & 1u;
+        if (!tab) {
+          const int ed = a.slot_edge[6 * n + s];
+          const bool isp = a.edge_pq[2 * ed] == n;
+          bool upp;
+          cs = side_prefactor<R>(cg, a.edge_geo + 8 * ed, upp);
+          if (!isp) cs = -cs;
+          upn = upp == isp;
+          if (upn && !AP && !AM) a_self[e] += cs;
+          cs = per_solid_angle(cs, a.dOmega, a.rdO, n);
         }
-        R sp = -(v0 * q0 + v1 * q1 + v2 * q2);          // V . nu (nu is normal to n_e)
-        R n0e = cg.M[0][0] + cg.M[0][1] * x + cg.M[0][2] * y + cg.M[0][3] * z;
-        R Pv = len * sp * n0e;
-        R PL = sp >= R(0) ? Pv : R(0), PR = sp >= R(0) ? R(0) : Pv;
-        R dOn = e ? dO_[1] : dO_[0];
-        const bool isp = a.edge_pq[2 * ed] == n;
         if (AP) {
           // the flux out of n through this side is cs times the upwind cell's
           // reconstruction at the side; kept: cs, and packed the neighbour m,
           // the cell of the upwind line beyond the side (behind n when n is
           // upwind, beyond m otherwise) and whether n is upwind
-          const bool upn = isp ? sp >= R(0) : sp < R(0);
+          const int ed = a.slot_edge[6 * n + s];
+          const bool isp = a.edge_pq[2 * ed] == n;
           const int *el = a.edge_line + 2 * ed;
           const int l = upn ? el[isp ? 0 : 1] : el[isp ? 1 : 0];
-          a_nb[e][s] = (isp ? Pv : -Pv) / dOn;
+          a_nb[e][s] = cs;
           nb_m[e][s] = m | (l << 12) | (upn ? 1 << 24 : 0);
         } else if (AM) {
           // as above, with the upwind cell's plane evaluated at the side's
           // midpoint (its gnomonic coordinates in that cell's tangent plane)
-          const bool upn = isp ? sp >= R(0) : sp < R(0);
-          a_nb[e][s] = (isp ? Pv : -Pv) / dOn;
+          a_nb[e][s] = cs;
           nb_m[e][s] = m | (upn ? 1 << 24 : 0);
           const double *xs = (upn ? a.mapr_xo : a.mapr_xn) + 12 * n + 2 * s;
           xu[e][s][0] = (R)xs[0];
           xu[e][s][1] = (R)xs[1];
-        } else if (isp) {
-          self += PL;
-          a_nb[e][s] = PR / dOn;
-        } else {
-          self -= PR;
-          a_nb[e][s] = -PL / dOn;
+        } else if (!upn) {
+          a_nb[e][s] = cs;
         }
       }
-      a_self[e] = ac ? self / (e ? dO_[1] : dO_[0]) : R(0);
+    }
+    if (!AP && !AM) {
+      const V sv = tab ? __ldg((const V *)(trow + kMaxSlots * nap)) : P::mk(R(0), R(0));
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+        if (b0 + e < a.nang) a_self[e] = tab ? (e ? sv.y : sv.x) : per_solid_angle(a_self[e], a.dOmega, a.rdO, b0 + e);
     }
   }
   // ---- stencil rows of one cell (h = 2, or 3 for PPM): the contiguous x1
