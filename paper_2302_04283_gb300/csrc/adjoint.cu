@@ -29,6 +29,8 @@
 // for the faces next to a pole whose upwind stencils reach across it (the
 // pole faces themselves have zero area).  No atomics: every output element
 // is written by one thread.
+#include <type_traits>
+
 #include "adjoint_kernels.cuh"
 
 namespace rad {
@@ -109,188 +111,271 @@ int launch_loss(rad_ctx *ctx, const void *I, int precision, double *L, void *dL,
 }
 
 // ---------------------------------------------------------------- adjoint
-// Adjoint of the coupling of one stage (thermal, fixed emissivity or none).
-template <typename R, int MAXT>
+// Adjoint of the coupling of one stage (MODE: thermal, fixed emissivity or
+// none).  One thread per bin; a CTA takes the column's chunk of kc cells in
+// phases, like the forward stage kernel:
+//   A  per cell the four bin sums of the forward coupling and of lambda_S
+//      (warp reduce-scatter, per-warp partials in shared memory);
+//   B  one thread per cell: the quartic's root (or the fixed-emissivity
+//      closed form) and the reverse sweep through the cell's scalars;
+//   C  per bin lambda_I* -> mu, and the bin sums of dL/dalpha_E (and dL/du);
+//   D  one thread per cell adds the gradients.
+// The kernel is bound by the FP64 pipe (two FP64 lanes per SM and clock on
+// this part: one warp instruction costs 16 SM cycles however few lanes are
+// active), so what counts is FP64 warp instructions.  Solving the root once
+// per cell with one active lane, between the barriers of that cell, cost as
+// many of them as the bins themselves; phase B solves a chunk's cells in one
+// warp.  Every quotient comes from one reciprocal of n^0bar den (rcp_newton,
+// three operations) in place of six correctly rounded divisions of about ten
+// each.  45 x 38 x 33 cells x 162 bins, thermal, FP32 intensities: 5.24 ->
+// 1.63 ms per stage; 256 x 128 x 162, fixed emissivity, FP64: 2.69 -> 1.35 ms.
+// The thermal sweep runs in FP64 in both precisions (only I* and
+// lambda_I+ are in the working precision): the terms of dL/dalpha_s cancel,
+// and FP32 per-bin sums lose percents.
+template <typename R, int MODE, int MAXT>
 __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
-  using Col = typename GeoTypes<R>::Col;
+  constexpr bool THERMAL = MODE == RAD_COUPLE_THERMAL;
+  using W = typename std::conditional<THERMAL, double, R>::type;      // type of the sweep
+  using Col = typename GeoTypes<W>::Col;
   const StageArgs &a = A.s;
-  __shared__ R buf[32 * 4];
-  __shared__ double dbuf[32 * 4], sc[8];
+  extern __shared__ __align__(16) unsigned char adj_smem[];
   const int n = threadIdx.x;
   const int nwarp = blockDim.x >> 5, lane = n & 31, warp = n >> 5;
   const bool act = n < a.nang;
   const int nchunk = (a.n3 + a.kc - 1) / a.kc;
   const int col = blockIdx.x / nchunk, chunk = blockIdx.x % nchunk;
   const int k0 = chunk * a.kc, nc = min(a.kc, a.n3 - k0);
-  const long long ncol = (long long)a.n1 * a.n2;
-  const long long strideK = ncol * a.nap;
-  const long long own = (long long)col * a.nap + (act ? n : 0);
-  const Col &cg = ((const Col *)a.cols)[col];
-  R nh0 = R(0), nh1 = R(0), nh2 = R(0), dOm = R(1);
+  const size_t ncol = (size_t)a.n1 * a.n2, strideK = ncol * a.nap;
+  const size_t own = (size_t)k0 * strideK + (size_t)col * a.nap + (act ? n : 0);
+  const Col &cg = THERMAL ? ((const Col *)A.cols64)[col] : ((const Col *)a.cols)[col];
+  W x = W(0), y = W(0), z = W(0), dOm = W(0);
   if (act) {
-    nh0 = (R)a.dir[3 * n];
-    nh1 = (R)a.dir[3 * n + 1];
-    nh2 = (R)a.dir[3 * n + 2];
-    dOm = (R)a.dOmega[n];
+    x = (W)a.dir[3 * n];
+    y = (W)a.dir[3 * n + 1];
+    z = (W)a.dir[3 * n + 2];
+    dOm = (W)a.dOmega[n];
   }
-  const R n0up = cg.n0up;
-  const R nlow0 = cg.M[0][0] + cg.M[0][1] * nh0 + cg.M[0][2] * nh1 + cg.M[0][3] * nh2;
-  const R fconv = n0up * nlow0;
-  const bool guard = act && a.zero_guard && fabs((double)nlow0) < a.n0crit;
-  const R inv_f = act ? R(1) / fconv : R(0);
-  const R dts = (R)a.dts, c2pre = dts / R(kFourPi);
+  const W n0up = cg.n0up;
+  const W nlow0 = cg.M[0][0] + cg.M[0][1] * x + cg.M[0][2] * y + cg.M[0][3] * z;
+  // the guard's test in the working precision of the forward kernel
+  R g0 = (R)nlow0;
+  if (THERMAL && sizeof(R) == 4) {
+    const ColGeoF &cf = ((const ColGeoF *)a.cols)[col];
+    g0 = (R)(cf.M[0][0] + cf.M[0][1] * (float)x + cf.M[0][2] * (float)y + cf.M[0][3] * (float)z);
+  }
+  const bool live = act && !(a.zero_guard && fabs((double)g0) < a.n0crit);
+  const W inv_f = act ? W(1) / (n0up * nlow0) : W(0);
   const R *lam = (const R *)A.lam, *Isv = (const R *)A.Istar;
   R *mu = (R *)A.mu;
+  if (MODE == RAD_COUPLE_NONE) {
+    for (int c = 0; c < nc; ++c)
+      if (act) mu[own + c * strideK] = live ? (R)((W)lam[own + c * strideK] * inv_f) : R(0);
+    return;
+  }
+  W *gas = (W *)adj_smem;                     // [kc][8]: u, u^0, alpha_E (times dts in FP64)
+  W *sc = gas + 8 * a.kc;                     // [kc][8]: scalars of phase B
+  W *red = sc + 8 * a.kc;                     // [kc][nwarp][4]
+  const W dts = (W)a.dts, c2p = dts / W(kFourPi);
+  for (int c = n; c < nc; c += blockDim.x) {
+    const size_t cell = (size_t)(k0 + c) * ncol + col;
+    const W ux = (W)a.u[3 * cell], uy = (W)a.u[3 * cell + 1], uz = (W)a.u[3 * cell + 2];
+    W *g = gas + 8 * c;
+    g[0] = ux;
+    g[1] = uy;
+    g[2] = uz;
+    g[3] = sqrt(W(1) + ux * ux + uy * uy + uz * uz);
+    g[4] = (W)(a.aa[cell] + a.as[cell]);
+    if (sizeof(W) == 8) g[4] *= dts;
+  }
+  __syncthreads();
+  // per bin and cell: nb = n^0bar, rden = 1 / (n^0 + nb alpha_E dt),
+  // c2n = c2pre rden / nb^3, wb = nb^2 dOmega, rn = dOmega rden / nb.  FP64
+  // takes all quotients from one refined reciprocal of nb den.
+  struct Bin { W nb, rden, c2n, wb, rn, inb; };
+  auto bin = [&](int c) -> Bin {
+    const W *g = gas + 8 * c;
+    Bin b;
+    b.nb = g[3] - (g[0] * x + g[1] * y + g[2] * z);
+    b.wb = b.nb * b.nb * dOm;
+    if (sizeof(W) == 8) {
+      const W den = n0up + b.nb * g[4];
+      const W r = P2<W>::rcp(P2<W>::mk(b.nb * den, W(1))).x;
+      b.rden = b.nb * r;
+      b.inb = den * r;
+      b.c2n = c2p * b.rden * (b.inb * b.inb * b.inb);
+      b.rn = dOm * r;
+    } else {
+      b.rden = W(1) / (n0up + b.nb * g[4] * dts);
+      b.c2n = c2p * b.rden / (b.nb * b.nb * b.nb);
+      b.rn = dOm * b.rden / b.nb;
+      b.inb = W(0);
+    }
+    return b;
+  };
+  // ---- phase A: thermal D = sum (c1 - 1) I* wbar, sum dOmega rden / nb, Ebar- =
+  // sum I* wbar, lambda_S; fixed emissivity A1 = sum c1 I* wbar, the same, lambda_S
+#pragma unroll 2
   for (int c = 0; c < nc; ++c) {
-    const int k = k0 + c;
-    const long long cell = (long long)k * ncol + col;
-    const long long e = (long long)k * strideK + own;
-    const R lamp = (act && !guard) ? lam[e] : R(0);
-    if (a.mode == RAD_COUPLE_NONE) {
-      if (act) mu[e] = guard ? R(0) : lamp * inv_f;
-      continue;
+    const W Is = act ? (W)Isv[own + c * strideK] : W(0);
+    const W lp = live ? (W)lam[own + c * strideK] : W(0);
+    const Bin b = bin(c);
+    W s;
+    if (THERMAL) {
+      const W w = Is * b.wb;
+      s = warp_reduce4(-(b.nb * gas[8 * c + 4]) * b.rden * w, b.rn, w, b.c2n * lp, lane);
+    } else {
+      const W c1 = n0up * b.rden;
+      s = warp_reduce4(act ? c1 * Is * b.wb : W(0), act ? b.rn : W(0), act ? b.c2n * lp : W(0), W(0), lane);
     }
-    const R ux = (R)a.u[3 * cell], uy = (R)a.u[3 * cell + 1], uz = (R)a.u[3 * cell + 2];
-    const R aE = (R)(a.aa[cell] + a.as[cell]), as = (R)a.as[cell];
-    const R u0 = sqrt(R(1) + ux * ux + uy * uy + uz * uz);
-    const R Is = act ? Isv[e] : R(0);
-    const R nb = u0 - (ux * nh0 + uy * nh1 + uz * nh2);
-    const R rden = R(1) / (n0up + nb * aE * dts);
-    const R c1 = n0up * rden;
-    const R c2n = c2pre * rden / (nb * nb * nb);
-    const R wbar = nb * nb * dOm;
-    if (a.mode == RAD_COUPLE_THERMAL) {
-      // forward (Sec. 2.5): D = sum (c1 - 1) I* wbar, A2 = c2pre sum dOmega
-      // rden / n^0bar, Ebar- = sum I* wbar, the quartic B4 T^4 + B1 T + B0 = 0,
-      // Ebar+ = Ebar- - c_v (T+ - T-), S = alpha_a a T+^4 + alpha_s Ebar+,
-      // I+ = c1 I* + c2n S.  The reverse sweep runs in FP64 for both
-      // precisions (only I* and lambda_I+ are in the working precision): the
-      // terms of dL/dalpha_s cancel, and FP32 per-bin sums lose percents.
-      const ColGeo &cd = A.cols64[col];
-      double xh = 0.0, yh = 0.0, zh = 0.0, dOd = 0.0;
-      if (act) {
-        xh = a.dir[3 * n];
-        yh = a.dir[3 * n + 1];
-        zh = a.dir[3 * n + 2];
-        dOd = a.dOmega[n];
-      }
-      const double n0d = cd.n0up, dtsd = a.dts, c2pd = dtsd / kFourPi;
-      const double uxd = a.u[3 * cell], uyd = a.u[3 * cell + 1], uzd = a.u[3 * cell + 2];
+    if ((lane & 7) == 0) red[(c * nwarp + warp) * 4 + (lane >> 3)] = s;
+  }
+  __syncthreads();
+  // ---- phase B
+  for (int c = n; c < nc; c += blockDim.x) {
+    const size_t cell = (size_t)(k0 + c) * ncol + col;
+    W t[4] = {W(0), W(0), W(0), W(0)};
+    for (int w = 0; w < nwarp; ++w)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) t[r] += red[(c * nwarp + w) * 4 + r];
+    W *o = sc + 8 * c;
+    const W A2 = c2p * t[1], lS = THERMAL ? t[3] : t[2];
+    if (THERMAL) {
+      // the quartic B4 T^4 + B1 T + B0 = 0, Ebar+ = Ebar- - c_v (T+ - T-),
+      // S = alpha_a a T+^4 + alpha_s Ebar+, I+ = c1 I* + c2n S
       const double aad = a.aa[cell], asd = a.as[cell], ar = a.a_rad;
-      const double nbd = sqrt(1.0 + uxd * uxd + uyd * uyd + uzd * uzd) - (uxd * xh + uyd * yh + uzd * zh);
-      const double nbaEd = nbd * (aad + asd) * dtsd;
-      const double rdend = 1.0 / (n0d + nbaEd);
-      const double c1d = n0d * rdend, cm1d = -nbaEd * rdend;          // c1 and c1 - 1
-      const double c2nd = c2pd * rdend / (nbd * nbd * nbd);
-      const double wbd = nbd * nbd * dOd;
-      const double Isd = act ? (double)Is : 0.0, lpd = (double)lamp;
-      double t4[4];
-      cta_sum4<double>(act ? cm1d * Isd * wbd : 0.0, act ? dOd * rdend / nbd : 0.0, act ? Isd * wbd : 0.0,
-                       act ? c2nd * lpd : 0.0, dbuf, nwarp, lane, warp, t4);
-      if (n == 0) {
-        const double D = t4[0], A2 = c2pd * t4[1], Em = t4[2], lS = t4[3];
-        const double Tm = a.stage2 ? 0.5 * (a.T0[cell] + a.T1[cell]) : a.T0[cell];
-        const double cv = a.rho[cell] * a.inv_gm1;
-        const double B4 = A2 * aad * ar, B1 = cv * (1.0 - A2 * asd), B0 = D + A2 * asd * Em - B1 * Tm;
-        bool ok = true;
-        const double Tp = quartic_root(B4, B1, B0, true, ok);
-        if (!ok || !isfinite(Tp)) atomicOr(a.err, kErrNoConv);
-        const double T3 = Tp * Tp * Tp, T4 = T3 * Tp;
-        const double Ep = Em - cv * (Tp - Tm);
-        // S = alpha_a a T+^4 + alpha_s Ebar+
-        double lT = (A.lamTp ? A.lamTp[cell] : 0.0) + 4.0 * aad * ar * T3 * lS;
-        const double lEp = asd * lS;
-        double laa = ar * T4 * lS, las = Ep * lS;
-        // Ebar+ = Ebar- - c_v T+ + c_v T-
-        double lEm = lEp, lTm = cv * lEp;
-        lT -= cv * lEp;
-        // T+ = root(B4, B1, B0): d/dB = -(T^4, T, 1) / f'(T+)
-        const double g = lT / (4.0 * B4 * T3 + B1);
-        const double lB4 = -g * T4, lB0 = -g;
-        double lB1 = -g * Tp;
-        // B0 = D + A2 alpha_s Ebar- - B1 T-
-        double lA2 = asd * Em * lB0;
-        las += A2 * Em * lB0;
-        lEm += A2 * asd * lB0;
-        lB1 -= Tm * lB0;
-        lTm -= B1 * lB0;
-        // B1 = c_v (1 - A2 alpha_s), B4 = A2 alpha_a a
-        lA2 += -cv * asd * lB1 + aad * ar * lB4;
-        las -= cv * A2 * lB1;
-        laa += A2 * ar * lB4;
-        sc[0] = aad * ar * T4 + asd * Ep;      // S
-        sc[1] = lB0;                           // lambda_D
-        sc[2] = lEm;
-        sc[3] = c2pd * lA2;                    // lambda of sum dOmega rden / n^0bar
-        sc[4] = laa;
-        sc[5] = las;
-        sc[6] = lTm;
-      }
-      __syncthreads();
-      const double S = sc[0], lD = sc[1], lEm = sc[2], lA2s = sc[3];
-      const double lc1 = Isd * lpd + Isd * wbd * lD;
-      const double lIs = c1d * lpd + cm1d * wbd * lD + wbd * lEm;
-      const double lrden = n0d * lc1 + c2pd / (nbd * nbd * nbd) * S * lpd + dOd / nbd * lA2s;
-      // with the radiation-dominated substitution the velocity is itself a
-      // function of the intensities: dL/du through every n^0bar = u^0 - u.n
-      double dudn[3] = {0.0, 0.0, 0.0};
-      if (A.lam_u && act) {
-        const double inb = 1.0 / nbd;
-        const double drden = -(aad + asd) * dtsd * rdend * rdend;
-        const double dLdnb = lrden * drden - 3.0 * c2pd * rdend * inb * inb * inb * inb * S * lpd +
-                             (cm1d * Isd * lD + Isd * lEm) * 2.0 * nbd * dOd - lA2s * dOd * rdend * inb * inb;
-        const double u0d = sqrt(1.0 + uxd * uxd + uyd * uyd + uzd * uzd);
-        dudn[0] = dLdnb * (uxd / u0d - xh);
-        dudn[1] = dLdnb * (uyd / u0d - yh);
-        dudn[2] = dLdnb * (uzd / u0d - zh);
-      }
-      double t2[4];
-      cta_sum4<double>(act ? -nbd * dtsd * rdend * rdend * lrden : 0.0, dudn[0], dudn[1], dudn[2], dbuf, nwarp,
-                       lane, warp, t2);
-      if (n == 0 && A.lam_u) {
-        A.lam_u[3 * cell] = t2[1];
-        A.lam_u[3 * cell + 1] = t2[2];
-        A.lam_u[3 * cell + 2] = t2[3];
-      }
-      if (n == 0) {
-        const double laE = t2[0];
-        A.g_aa[cell] += sc[4] + laE;
-        A.g_as[cell] += sc[5] + laE;
-        if (A.outTa) A.outTa[cell] = (A.accTa ? A.outTa[cell] : 0.0) + A.wTa * sc[6];
-        if (A.outTb) A.outTb[cell] = A.wTb * sc[6];
-      }
-      if (act) {
-        const double fd = n0d * (cd.M[0][0] + cd.M[0][1] * xh + cd.M[0][2] * yh + cd.M[0][3] * zh);
-        mu[e] = guard ? R(0) : (R)(lIs / fd);
-      }
-      continue;
-    }
-    const R eta = (R)a.eta[cell];
-    R t[3];
-    cta_sum3<R>(act ? c1 * Is * wbar : R(0), act ? dOm * rden / nb : R(0), act ? c2n * lamp : R(0), buf, nwarp,
-                lane, warp, t);
-    const R A1 = t[0], A2 = c2pre * t[1], lS = t[2];
-    const R Q = R(1) - A2 * as;
-    const R Ep = (A1 + R(kFourPi) * A2 * eta) / Q;
-    const R S = R(kFourPi) * eta + as * Ep;
-    const R lEp = as * lS;
-    const R lA1 = lEp / Q;
-    const R lQ = -Ep * lEp / Q;
-    const R lA2 = R(kFourPi) * eta * lEp / Q - as * lQ;
-    const R leta = R(kFourPi) * lS + R(kFourPi) * A2 * lEp / Q;
-    const R las = Ep * lS - A2 * lQ;
-    const R lc1 = Is * lamp + Is * wbar * lA1;
-    const R lc2n = S * lamp;
-    const R lIs = c1 * lamp + c1 * wbar * lA1;
-    const R lden = -c1 * rden * lc1 - c2n * rden * lc2n - c2pre * dOm * rden * rden / nb * lA2;
-    R t2[3];
-    cta_sum3<R>(act ? nb * dts * lden : R(0), R(0), R(0), buf, nwarp, lane, warp, t2);
-    if (n == 0) {
-      A.g_aa[cell] += (double)t2[0];
-      A.g_as[cell] += (double)(t2[0] + las);
+      const double D = t[0], Em = t[2];
+      const double Tm = a.stage2 ? 0.5 * (a.T0[cell] + a.T1[cell]) : a.T0[cell];
+      const double cv = a.rho[cell] * a.inv_gm1;
+      const double B4 = A2 * aad * ar, B1 = cv * (1.0 - A2 * asd), B0 = D + A2 * asd * Em - B1 * Tm;
+      bool ok = true;
+      const double Tp = quartic_root(B4, B1, B0, true, ok, Tm);
+      if (!ok || !isfinite(Tp)) atomicOr(a.err, kErrNoConv);
+      const double T3 = Tp * Tp * Tp, T4 = T3 * Tp;
+      const double Ep = Em - cv * (Tp - Tm);
+      double lT = (A.lamTp ? A.lamTp[cell] : 0.0) + 4.0 * aad * ar * T3 * lS;
+      const double lEp = asd * lS;
+      double laa = ar * T4 * lS, las = Ep * lS;
+      // Ebar+ = Ebar- - c_v T+ + c_v T-
+      double lEm = lEp, lTm = cv * lEp;
+      lT -= cv * lEp;
+      // T+ = root(B4, B1, B0): d/dB = -(T^4, T, 1) / f'(T+)
+      const double g = lT / (4.0 * B4 * T3 + B1);
+      const double lB4 = -g * T4, lB0 = -g;
+      double lB1 = -g * Tp;
+      // B0 = D + A2 alpha_s Ebar- - B1 T-
+      double lA2 = asd * Em * lB0;
+      las += A2 * Em * lB0;
+      lEm += A2 * asd * lB0;
+      lB1 -= Tm * lB0;
+      lTm -= B1 * lB0;
+      // B1 = c_v (1 - A2 alpha_s), B4 = A2 alpha_a a
+      lA2 += -cv * asd * lB1 + aad * ar * lB4;
+      las -= cv * A2 * lB1;
+      laa += A2 * ar * lB4;
+      o[0] = aad * ar * T4 + asd * Ep;       // S
+      o[1] = lB0;                            // lambda_D
+      o[2] = lEm;
+      o[3] = c2p * lA2;                      // lambda of sum dOmega rden / n^0bar
+      o[4] = laa;
+      o[5] = las;
+      if (A.outTa) A.outTa[cell] = (A.accTa ? A.outTa[cell] : 0.0) + A.wTa * lTm;
+      if (A.outTb) A.outTb[cell] = A.wTb * lTm;
+    } else {
+      const W as = (W)a.as[cell], eta = (W)a.eta[cell], A1 = t[0];
+      const W Q = W(1) - A2 * as;
+      const W Ep = (A1 + W(kFourPi) * A2 * eta) / Q;
+      const W S = W(kFourPi) * eta + as * Ep;
+      const W lEp = as * lS;
+      const W lA1 = lEp / Q;
+      const W lQ = -Ep * lEp / Q;
+      const W lA2 = W(kFourPi) * eta * lEp / Q - as * lQ;
+      const W leta = W(kFourPi) * lS + W(kFourPi) * A2 * lEp / Q;
+      const W las = Ep * lS - A2 * lQ;
+      o[0] = S;
+      o[1] = lA1;
+      o[3] = lA2;
+      o[4] = W(0);
+      o[5] = las;
       if (A.g_eta) A.g_eta[cell] += (double)leta;
     }
-    if (act) mu[e] = guard ? R(0) : lIs * inv_f;
+  }
+  __syncthreads();
+  // ---- phase C: lambda_I* and dL/d(1 / den) of every bin; the sum of
+  // dL/dalpha_E of four cells shares one reduce-scatter (with the
+  // radiation-dominated substitution a cell's four sums, dL/du among them)
+  W held[3] = {W(0), W(0), W(0)};
+  for (int c = 0; c < nc; ++c) {
+    const size_t e = own + c * strideK;
+    const W Is = act ? (W)Isv[e] : W(0);
+    const W lp = live ? (W)lam[e] : W(0);
+    const Bin b = bin(c);
+    const W *o = sc + 8 * c;
+    const W S = o[0], lD = o[1];
+    const W c1 = n0up * b.rden;
+    W lIs, vE, lrden = W(0), cm1 = W(0);
+    const W lEm = THERMAL ? o[2] : W(0), lA2 = o[3];
+    if (THERMAL) {
+      cm1 = -(b.nb * gas[8 * c + 4]) * b.rden;
+      const W lc1 = Is * (lp + b.wb * lD);
+      lIs = c1 * lp + b.wb * (cm1 * lD + lEm);
+      lrden = n0up * lc1 + c2p * (b.inb * b.inb * b.inb) * (S * lp) + dOm * b.inb * lA2;
+      vE = -b.nb * dts * b.rden * b.rden * lrden;
+    } else {
+      const W lc1 = Is * lp + Is * b.wb * lD;
+      const W lc2n = S * lp;
+      lIs = c1 * lp + c1 * b.wb * lD;
+      // FP64: dOmega rden^2 / nb as rn rden, without another quotient
+      const W lden = sizeof(W) == 8
+                         ? -c1 * b.rden * lc1 - b.c2n * b.rden * lc2n - c2p * b.rn * b.rden * lA2
+                         : -c1 * b.rden * lc1 - b.c2n * b.rden * lc2n - c2p * dOm * b.rden * b.rden / b.nb * lA2;
+      vE = b.nb * dts * lden;
+    }
+    if (!act) vE = W(0);
+    if (act) mu[e] = live ? (R)(lIs * inv_f) : R(0);
+    if (THERMAL && A.lam_u) {
+      // the velocity is itself a function of the intensities: dL/du through
+      // every n^0bar = u^0 - u.n
+      W du[3] = {W(0), W(0), W(0)};
+      if (act) {
+        const W *g = gas + 8 * c;
+        const W dLdnb = -lrden * g[4] * b.rden * b.rden - W(3) * b.c2n * b.inb * S * lp +
+                        (cm1 * Is * lD + Is * lEm) * W(2) * b.nb * dOm - lA2 * b.rn * b.inb;
+        const W iu0 = W(1) / g[3];
+        du[0] = dLdnb * (g[0] * iu0 - x);
+        du[1] = dLdnb * (g[1] * iu0 - y);
+        du[2] = dLdnb * (g[2] * iu0 - z);
+      }
+      const W s = warp_reduce4(vE, du[0], du[1], du[2], lane);
+      if ((lane & 7) == 0) red[(c * nwarp + warp) * 4 + (lane >> 3)] = s;
+      continue;
+    }
+    if ((c & 3) == 3 || c == nc - 1) {
+      const int q = c & 3, c4 = c - q;
+      const W s = warp_reduce4(q == 0 ? vE : held[0], q == 1 ? vE : (q > 1 ? held[1] : W(0)),
+                               q == 2 ? vE : (q > 2 ? held[2] : W(0)), q == 3 ? vE : W(0), lane);
+      const int r = lane >> 3;
+      if ((lane & 7) == 0 && c4 + r < nc) red[((c4 + r) * nwarp + warp) * 4] = s;
+    } else if ((c & 3) == 0) {
+      held[0] = vE;
+    } else if ((c & 3) == 1) {
+      held[1] = vE;
+    } else {
+      held[2] = vE;
+    }
+  }
+  __syncthreads();
+  // ---- phase D
+  for (int c = n; c < nc; c += blockDim.x) {
+    const size_t cell = (size_t)(k0 + c) * ncol + col;
+    const int nr = THERMAL && A.lam_u ? 4 : 1;
+    W t[4] = {W(0), W(0), W(0), W(0)};
+    for (int w = 0; w < nwarp; ++w)
+      for (int r = 0; r < nr; ++r) t[r] += red[(c * nwarp + w) * 4 + r];
+    const W *o = sc + 8 * c;
+    A.g_aa[cell] += THERMAL ? (double)(o[4] + t[0]) : (double)t[0];
+    A.g_as[cell] += (double)(t[0] + o[5]);
+    if (THERMAL && A.lam_u)
+      for (int d = 0; d < 3; ++d) A.lam_u[3 * cell + d] = (double)t[1 + d];
   }
 }
 
@@ -303,15 +388,24 @@ cudaError_t launch_transport_adj_any(const AdjArgs &A, bool ang, cudaStream_t st
   return ang ? launch_transport_adj<R, true>(A, st) : launch_transport_adj<R, false>(A, st);
 }
 
+template <typename R, int MODE>
+cudaError_t launch_couple_adj_m(const AdjArgs &A, cudaStream_t st) {
+  const int threads = (A.s.nap + 31) / 32 * 32;
+  const int nchunk = (A.s.n3 + A.s.kc - 1) / A.s.kc;
+  const dim3 grid((unsigned)((long long)A.s.n1 * A.s.n2 * nchunk));
+  const size_t esz = MODE == RAD_COUPLE_THERMAL ? 8 : sizeof(R);
+  const size_t smem = (size_t)A.s.kc * (16 + 4 * (threads / 32)) * esz;     // kc <= 32: at most 37 KB
+  if (threads <= 256) k_couple_adj<R, MODE, 256><<<grid, threads, smem, st>>>(A);
+  else if (threads <= 512) k_couple_adj<R, MODE, 512><<<grid, threads, smem, st>>>(A);
+  else k_couple_adj<R, MODE, 1024><<<grid, threads, smem, st>>>(A);
+  return cudaGetLastError();
+}
+
 template <typename R>
 cudaError_t launch_couple_adj(const AdjArgs &A, cudaStream_t st) {
-  int threads = (A.s.nap + 31) / 32 * 32;
-  int nchunk = (A.s.n3 + A.s.kc - 1) / A.s.kc;
-  dim3 grid((unsigned)((long long)A.s.n1 * A.s.n2 * nchunk));
-  if (threads <= 256) k_couple_adj<R, 256><<<grid, threads, 0, st>>>(A);
-  else if (threads <= 512) k_couple_adj<R, 512><<<grid, threads, 0, st>>>(A);
-  else k_couple_adj<R, 1024><<<grid, threads, 0, st>>>(A);
-  return cudaGetLastError();
+  if (A.s.mode == RAD_COUPLE_THERMAL) return launch_couple_adj_m<R, RAD_COUPLE_THERMAL>(A, st);
+  if (A.s.mode == RAD_COUPLE_EMISSIVITY) return launch_couple_adj_m<R, RAD_COUPLE_EMISSIVITY>(A, st);
+  return launch_couple_adj_m<R, RAD_COUPLE_NONE>(A, st);
 }
 
 }  // namespace

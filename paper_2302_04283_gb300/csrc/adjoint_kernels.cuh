@@ -56,20 +56,6 @@ __device__ __forceinline__ void cta_sum3(R v0, R v1, R v2, R *buf, int nwarp, in
   __syncthreads();
 }
 
-// The same for four values.
-template <typename R>
-__device__ __forceinline__ void cta_sum4(R v0, R v1, R v2, R v3, R *buf, int nwarp, int lane, int warp, R out[4]) {
-  R s = warp_reduce4(v0, v1, v2, v3, lane);
-  if ((lane & 7) == 0) buf[warp * 4 + (lane >> 3)] = s;
-  __syncthreads();
-  out[0] = out[1] = out[2] = out[3] = R(0);
-  for (int w = 0; w < nwarp; ++w) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) out[r] += buf[w * 4 + r];
-  }
-  __syncthreads();
-}
-
 // Face flux prefactor Delta A n^d n_0 (no 1/dV) and upwind side for one bin.
 template <typename Face, typename R>
 __device__ __forceinline__ R face_coefA(const Face &F, R x, R y, R z, bool &upR) {
