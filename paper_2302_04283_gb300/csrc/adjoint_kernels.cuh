@@ -38,6 +38,9 @@ struct AdjArgs {
   // radiation-dominated substitution: the coupling runs at the substituted
   // velocity (s.u points at it) and writes dL/du [cell][3] here (nullable)
   double *lam_u;
+  // transport adjoint: the inner cells are k_transport_adj_in's, this kernel
+  // takes the others
+  int split;
 };
 
 // Three-value CTA reduction used per cell: warp reduce-scatter, then every
@@ -168,6 +171,19 @@ __device__ __forceinline__ void edge_grad(bool plm, bool right, const R *w, R &p
   }
 }
 
+// Cells whose PLM / DC stencils reach no ghost: two cells from every face that
+// is not periodic, or anywhere on a periodic line of five cells or more (on a
+// shorter one a face can hold the cell twice).
+__device__ __forceinline__ bool adj_inner_1d(int x, int n, int bc_lo) {
+  return bc_lo == RAD_BC_PERIODIC ? n >= 5 : x >= 2 && x <= n - 3;
+}
+__device__ __forceinline__ bool adj_inner_column(const StageArgs &a, int i, int j) {
+  return adj_inner_1d(i, a.n1, a.bc_lo[0]) && (a.ndim < 2 || adj_inner_1d(j, a.n2, a.bc_lo[1]));
+}
+__device__ __forceinline__ bool adj_inner_k(const StageArgs &a, int k) {
+  return a.ndim < 3 || adj_inner_1d(k, a.n3, a.bc_lo[2]);
+}
+
 // Transposed angular coefficients of bin n in a column (donor cell): what
 // divA of the bin itself and of its neighbours take from I_n.  With c_s the
 // prefactor of the flux out of n through side s, divA_n = sum_s c_s
@@ -205,6 +221,209 @@ __device__ __forceinline__ void side_transposed(const StageArgs &a, const Col &c
   }
 }
 
+// Gradient of the half-slope q(v0, v1, v2) in its three cells, zero unless the
+// slope's product is positive: -(dr/s)^2, (dr^2 - dl^2)/s^2, (dl/s)^2.  FP32
+// takes dphi's operations; FP64 forms them from one refined reciprocal of s
+// (a correctly rounded division costs ten operations of the FP64 pipe).
+__device__ __forceinline__ void slope_grad_of(float dl, float dr, float d[3]) {
+  const float s = dl + dr, is2 = 1.0f / (s * s);
+  d[0] = -dr * dr * is2;
+  d[1] = mul_rn(fma_rn(dr, dr, -mul_rn(dl, dl)), is2);      // rounded before it meets 1, as in dphi
+  d[2] = dl * dl * is2;
+}
+__device__ __forceinline__ void slope_grad_of(double dl, double dr, double d[3]) {
+  const double r = rcp_newton(dl + dr), a = dr * r, b = dl * r;
+  d[0] = -a * a;
+  d[1] = a - b;
+  d[2] = b * b;
+}
+template <typename R>
+__device__ __forceinline__ void slope_grad(R v0, R v1, R v2, R d[3]) {
+  const R dl = v1 - v0, dr = v2 - v1;
+  d[0] = d[1] = d[2] = R(0);
+  if (dl * dr > R(0)) slope_grad_of(dl, dr, d);
+}
+
+// Transposed transport of the inner cells (adj_inner_*) for DC and PLM
+// without the optical-depth weighting and with donor-cell angular fluxes; the
+// general kernel below takes the cells next to the boundaries and every other
+// option, in the same order of operations.  Per dimension the cell appears in
+// three slopes (of the cells at -1, 0, 1) and in the four faces around them:
+// three gradients and four face weights, where the general form
+// differentiates four face states with two divisions each and sends every
+// window value through the boundary map.  x3 values ride in a register
+// window.  Bound by the FP64 pipe in FP64 and by the loads' latency in FP32;
+// one thread per bin, because 92 bins fill three warps of threads (96 %) but
+// two of pairs (72 %).  256 x 128 cells x 162 bins FP64 4.0 -> 2.0 ms per stage
+// (11.2 before the side table), 45 x 38 x 33 x 162 FP32 1.40 -> 0.74 ms.
+template <typename R, bool ANG>
+__global__ void __launch_bounds__(sizeof(R) == 8 ? 512 : 832) k_transport_adj_in(AdjArgs A) {
+  using Col = typename GeoTypes<R>::Col;
+  using Face = typename GeoTypes<R>::Face;
+  const StageArgs &a = A.s;
+  const int nchunk = (a.n3 + a.kc - 1) / a.kc;
+  const int col = blockIdx.x / nchunk, chunk = blockIdx.x % nchunk;
+  const int i = col % a.n1, j = col / a.n1;
+  if (!adj_inner_column(a, i, j)) return;
+  const int n = threadIdx.x;
+  const bool act = n < a.nang;
+  const int k0 = chunk * a.kc, nc = min(a.kc, a.n3 - k0);
+  const unsigned ncol = (unsigned)a.n1 * a.n2, strideK = ncol * (unsigned)a.nap;   // 32-bit offsets (host-checked)
+  const bool plm = a.recon == RAD_RECON_PLM;
+  const R *Il = (const R *)A.Ilin, *mu = (const R *)A.mu;
+  const Col *cols = (const Col *)a.cols;
+  const int bn = act ? n : 0;
+  R x = R(0), y = R(0), z = R(0);
+  if (act) {
+    x = (R)a.dir[3 * n];
+    y = (R)a.dir[3 * n + 1];
+    z = (R)a.dir[3 * n + 2];
+  }
+  const Col &cg = cols[col];
+  const R fconv = cg.n0up * (cg.M[0][0] + cg.M[0][1] * x + cg.M[0][2] * y + cg.M[0][3] * z);
+  // prefactors and upwind sides of the four faces of each dimension; rows and
+  // 1/dV at -2 .. 2
+  R cA[3][4], iv[3][5];
+  unsigned off[2][5], up[3] = {0u, 0u, 0u};
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    const int N = d == 0 ? a.n1 : a.n2, yd = d == 0 ? i : j;
+#pragma unroll
+    for (int t = 0; t < 5; ++t) {
+      iv[d][t] = R(0);
+      off[d][t] = 0u;
+      if (d >= a.ndim) continue;
+      int p = yd + t - 2;
+      p = p < 0 ? p + N : (p >= N ? p - N : p);
+      const int c2 = d == 0 ? j * a.n1 + p : p * a.n1 + i;
+      iv[d][t] = cols[c2].invdV;
+      off[d][t] = (unsigned)c2 * a.nap + bn;
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      cA[d][t] = R(0);
+      if (d >= a.ndim || !act) continue;
+      int f = yd + t - 1;                       // face between positions t - 2 and t - 1
+      f = f < 0 ? f + N : (f >= N && a.bc_lo[d] == RAD_BC_PERIODIC ? f - N : f);
+      const Face &F = d == 0 ? ((const Face *)a.f1)[j * (a.n1 + 1) + f] : ((const Face *)a.f2)[f * a.n1 + i];
+      bool u;
+      cA[d][t] = face_coefA(F, x, y, z, u);
+      up[d] |= (u ? 1u : 0u) << t;
+    }
+  }
+  {
+    bool u = false;
+    const R c = (act && a.ndim >= 3) ? face_coefA(((const Face *)a.f3)[col], x, y, z, u) : R(0);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) cA[2][t] = c;
+#pragma unroll
+    for (int t = 0; t < 5; ++t) iv[2][t] = cg.invdV;
+    up[2] = u ? 15u : 0u;
+  }
+  R at_self = R(0), at_nb[kMaxSlots];
+  int nb_m[kMaxSlots];
+  if (ANG) side_transposed<R>(a, cg, col, n, act, at_self, at_nb, nb_m);
+
+  // lambda through the faces of one dimension: values v and mu at -2 .. 2
+  auto dim = [&](int d, const R (&v)[5], const R (&mm)[5], const R (&ivd)[5], R lam) -> R {
+    const bool u0 = up[d] & 1, u1 = up[d] & 2, u2 = up[d] & 4, u3 = up[d] & 8;
+    R dm[3], d0[3], dp[3];         // gradients of the half-slopes of the cells at -1, 0, 1
+#pragma unroll
+    for (int q = 0; q < 3; ++q) dm[q] = d0[q] = dp[q] = R(0);
+    if (plm) {
+      slope_grad<R>(v[0], v[1], v[2], dm);
+      slope_grad<R>(v[1], v[2], v[3], d0);
+      slope_grad<R>(v[2], v[3], v[4], dp);
+    }
+    R lp[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      lp[t] = fma_rn(mul_rn(cA[d][t], ivd[t + 1]), mm[t + 1], mul_rn(mul_rn(-cA[d][t], ivd[t]), mm[t]));
+    }
+    // face 0 holds the cell only in the slope of its right cell, face 3 only
+    // in that of its left one
+    lam += lp[0] * (u0 ? -dm[2] : R(0));
+    lam += lp[1] * (u1 ? R(1) - d0[1] : dm[2]);
+    lam += lp[2] * (u2 ? -dp[0] : R(1) + d0[1]);
+    lam += lp[3] * (u3 ? R(0) : dp[0]);
+    return lam;
+  };
+  const bool d3 = a.ndim >= 3;
+  const unsigned own = (unsigned)col * a.nap + bn;
+  auto kidx = [&](int k) {      // periodic wrap; elsewhere the window's values beyond the line are not used
+    if (k >= 0 && k < a.n3) return k;
+    if (a.bc_lo[2] != RAD_BC_PERIODIC) return k < 0 ? 0 : a.n3 - 1;
+    k %= a.n3;
+    return k < 0 ? k + a.n3 : k;
+  };
+  R w[5], m[5];
+#pragma unroll
+  for (int q = 0; q < 5; ++q) w[q] = m[q] = R(0);
+  if (d3) {
+#pragma unroll
+    for (int q = 1; q < 5; ++q) {
+      const unsigned e = (unsigned)kidx(k0 - 3 + q) * strideK + own;
+      w[q] = Il[e];
+      m[q] = mu[e];
+    }
+  }
+  R *outA = (R *)A.outA, *outB = (R *)A.outB;
+  const R wAf = (R)A.wAf, wAL = (R)A.wAL, wBf = (R)A.wBf;
+  for (int c = 0; c < nc; ++c) {
+    const int k = k0 + c;
+    const unsigned base = (unsigned)k * strideK;
+    const R *I = Il + base, *M = mu + base;
+    if (d3) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        w[q] = w[q + 1];
+        m[q] = m[q + 1];
+      }
+      const unsigned e = (unsigned)kidx(k + 2) * strideK + own;
+      w[4] = Il[e];
+      m[4] = mu[e];
+      if (!adj_inner_k(a, k)) continue;
+    } else {
+      w[2] = I[own];
+      m[2] = M[own];
+    }
+    const R mu0 = m[2];
+    R lam = R(0);
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+      if (d >= a.ndim) continue;
+      R v[5], mm[5];
+#pragma unroll
+      for (int q = 0; q < 5; ++q) {
+        v[q] = q == 2 ? w[2] : (plm ? I[off[d][q]] : R(0));
+        mm[q] = q == 2 ? mu0 : M[off[d][q]];
+      }
+      lam = dim(d, v, mm, iv[d], lam);
+    }
+    if (d3) lam = dim(2, w, m, iv[2], lam);
+    if (ANG) {
+      R ga = at_self * mu0;
+#pragma unroll
+      for (int s = 0; s < kMaxSlots; ++s) ga += at_nb[s] * M[(unsigned)col * a.nap + nb_m[s]];
+      lam -= ga;
+    }
+    if (n < a.nap) {            // padding bins get zeros
+      const unsigned e = base + (unsigned)col * a.nap + n;
+      if (!act) {
+        outA[e] = R(0);
+        if (outB) outB[e] = R(0);
+        continue;
+      }
+      const R ra = fma_rn(mul_rn(wAf, fconv), mu0, mul_rn(wAL, lam));
+      outA[e] = A.accA ? outA[e] + ra : ra;
+      if (outB) {
+        const R rb = wBf * fconv * mu0;
+        outB[e] = A.accB ? outB[e] + rb : rb;
+      }
+    }
+  }
+}
+
 // Transposed transport of one stage (gather form, one thread per target bin).
 // PPM: the spatial reconstruction is PPM (each face state depends on the five
 // cells around its upwind cell) instead of DC / PLM (three cells).
@@ -226,6 +445,12 @@ __global__ void __launch_bounds__(MAXT, sizeof(R) == 8 ? 1 : 1280 / MAXT) k_tran
   const int col = blockIdx.x / nchunk, chunk = blockIdx.x % nchunk;
   const int i = col % a.n1, j = col / a.n1;
   const int k0 = chunk * a.kc, nc = min(a.kc, a.n3 - k0);
+  const bool colin = A.split && adj_inner_column(a, i, j);     // x1 and x2 are inner: k decides per cell
+  if (colin) {
+    bool all = true;
+    for (int c = 0; c < nc; ++c) all &= adj_inner_k(a, k0 + c);
+    if (all) return;
+  }
   const long long ncol = (long long)a.n1 * a.n2;
   const long long strideK = ncol * a.nap;
   const bool plm = a.recon == RAD_RECON_PLM;
@@ -376,6 +601,7 @@ __global__ void __launch_bounds__(MAXT, sizeof(R) == 8 ? 1 : 1280 / MAXT) k_tran
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   for (int c = 0; c < nc; ++c) {
     const int k = k0 + c;
+    if (colin && adj_inner_k(a, k)) continue;
     y[2] = k;
     R gt[3] = {R(0), R(0), R(0)};   // lower-face sums of this bin (optical-depth weighting)
     auto addr = [&](int ii, int jj, int kk, int bin) -> long long {
@@ -596,6 +822,9 @@ __global__ void __launch_bounds__(MAXT, sizeof(R) == 8 ? 1 : 1280 / MAXT) k_tran
         R rb = (R)A.wBf * fconv * mu0;
         outB[eown] = A.accB ? outB[eown] + rb : rb;
       }
+    } else if (n < a.nap) {     // padding bins get zeros
+      outA[addr(i, j, k, n)] = R(0);
+      if (outB) outB[addr(i, j, k, n)] = R(0);
     }
   }
 }
@@ -642,11 +871,18 @@ void launch_tadj(const AdjArgs &A, bool tau, bool ppm, dim3 grid, int threads, c
 
 // AR: angular reconstruction (curved space only): 0 donor cell, 1 line PLM, 2 MAPR
 template <typename R, bool ANG, int AR = 0>
-cudaError_t launch_transport_adj(const AdjArgs &A, cudaStream_t st) {
+cudaError_t launch_transport_adj(const AdjArgs &A0, cudaStream_t st) {
+  AdjArgs A = A0;
   int threads = (A.s.nap + 31) / 32 * 32;
   int nchunk = (A.s.n3 + A.s.kc - 1) / A.s.kc;
   dim3 grid((unsigned)((long long)A.s.n1 * A.s.n2 * nchunk));
   const bool tau = A.s.tau_const > 0.0, ppm = A.s.recon == RAD_RECON_PPM;
+  // inner cells of the plain DC / PLM form first (an FP64 CTA of more than
+  // 512 threads would not hold the kernel's registers: general form)
+  A.split = AR == 0 && !tau && !ppm && threads <= (sizeof(R) == 8 ? 512 : 832);
+  if constexpr (AR == 0) {
+    if (A.split) k_transport_adj_in<R, ANG><<<grid, threads, 0, st>>>(A);
+  }
   if (threads <= 256) launch_tadj<R, ANG, AR, 256>(A, tau, ppm, grid, threads, st);
   else if (threads <= 512) launch_tadj<R, ANG, AR, 512>(A, tau, ppm, grid, threads, st);
   else launch_tadj<R, ANG, AR, 1024>(A, tau, ppm, grid, threads, st);
