@@ -125,9 +125,8 @@ int launch_loss(rad_ctx *ctx, const void *I, int precision, double *L, void *dL,
 // active), so what counts is FP64 warp instructions.  Solving the root once
 // per cell with one active lane, between the barriers of that cell, cost as
 // many of them as the bins themselves; phase B solves a chunk's cells in one
-// warp.  Every quotient comes from one reciprocal of n^0bar den (rcp_newton,
-// three operations) in place of six correctly rounded divisions of about ten
-// each.  45 x 38 x 33 cells x 162 bins, thermal, FP32 intensities: 5.24 ->
+// warp.  Every quotient comes from one reciprocal of n^0bar den in place of
+// six correctly rounded divisions of about ten FP64 operations each.  45 x 38 x 33 cells x 162 bins, thermal, FP32 intensities: 5.24 ->
 // 1.63 ms per stage; 256 x 128 x 162, fixed emissivity, FP64: 2.69 -> 1.35 ms.
 // The thermal sweep runs in FP64 in both precisions (only I* and
 // lambda_I+ are in the working precision): the terms of dL/dalpha_s cancel,
@@ -190,7 +189,7 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
   __syncthreads();
   // per bin and cell: nb = n^0bar, rden = 1 / (n^0 + nb alpha_E dt),
   // c2n = c2pre rden / nb^3, wb = nb^2 dOmega, rn = dOmega rden / nb.  FP64
-  // takes all quotients from one refined reciprocal of nb den.
+  // takes all quotients from one reciprocal of nb den.
   struct Bin { W nb, rden, c2n, wb, rn, inb; };
   auto bin = [&](int c) -> Bin {
     const W *g = gas + 8 * c;

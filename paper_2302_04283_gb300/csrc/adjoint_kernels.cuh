@@ -223,8 +223,8 @@ __device__ __forceinline__ void side_transposed(const StageArgs &a, const Col &c
 
 // Gradient of the half-slope q(v0, v1, v2) in its three cells, zero unless the
 // slope's product is positive: -(dr/s)^2, (dr^2 - dl^2)/s^2, (dl/s)^2.  FP32
-// takes dphi's operations; FP64 forms them from one refined reciprocal of s
-// (a correctly rounded division costs ten operations of the FP64 pipe).
+// takes dphi's operations; FP64 forms them from one reciprocal of s (a
+// correctly rounded division costs ten operations of the FP64 pipe).
 __device__ __forceinline__ void slope_grad_of(float dl, float dr, float d[3]) {
   const float s = dl + dr, is2 = 1.0f / (s * s);
   d[0] = -dr * dr * is2;
@@ -232,7 +232,7 @@ __device__ __forceinline__ void slope_grad_of(float dl, float dr, float d[3]) {
   d[2] = dl * dl * is2;
 }
 __device__ __forceinline__ void slope_grad_of(double dl, double dr, double d[3]) {
-  const double r = rcp_newton(dl + dr), a = dr * r, b = dl * r;
+  const double r = rcp_digits(dl + dr), a = dr * r, b = dl * r;
   d[0] = -a * a;
   d[1] = a - b;
   d[2] = b * b;

@@ -43,6 +43,7 @@
 
 #include <string>
 
+#include "quotient.cuh"
 #include "rad_internal.h"
 #include "sides.cuh"
 
@@ -138,37 +139,15 @@ __device__ __forceinline__ float rcp_approx(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-// FP64 reciprocal: the hardware approximation r refined by one third-order
-// step.  With e = 1 - x r, 1/x = r / (1 - e) = r (1 + e + e^2 + ...); keeping
-// three terms, r <- r + r (e + e^2), turns a relative error eps of r into
-// about eps^3.  The approximation's eps measured on GB300 is below 1e-6
-// (2^-19.9 over 4M random x across the exponent range), so one step lands
-// within an ulp of the correctly rounded 1/x (equal to it for 99.97 % of
-// those x; two Newton-Raphson steps matched it everywhere).  Three FP64
-// operations instead of the four of two Newton-Raphson steps, and far
-// cheaper on the FP64 pipe than a correctly rounded division; far inside the
-// FP64 path's 1e-12 tolerance.  x = 0 gives a non-finite result (as 1/x
-// does); callers discard it.
-__device__ __forceinline__ double rcp_newton(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-// prod > 0 for the limiter: the FP32 compare, or in FP64 an integer test of
-// the high word (sign, exponent and the top of the mantissa), which keeps the
-// compare off the FP64 pipe.  A positive FP64 value whose high word is zero
-// (below 2^-1022 x 2^-20) counts as zero, so its limited slope, smaller
-// still, becomes zero.
-__device__ __forceinline__ bool pos_for_limiter(float v) { return v > 0.0f; }
-__device__ __forceinline__ bool pos_for_limiter(double v) { return __double2hiint(v) > 0; }
-
 // PLM half-slope q = dl dr / (dl + dr) if dl dr > 0 else 0 (van Leer 1974).
 template <typename R>
 __device__ __forceinline__ R vl_half(R x, R y, R z) {
   R dl = y - x, dr = z - y;
   R prod = dl * dr;
   return prod > R(0) ? fdiv(prod, dl + dr) : R(0);
+}
+template <> __device__ __forceinline__ double vl_half<double>(double x, double y, double z) {
+  return van_leer_digits(y - x, z - y);
 }
 
 // Upwind value at the face between cells b and c of the stencil a b | c d:
@@ -450,7 +429,7 @@ template <> struct P2<double> {
   static __device__ __forceinline__ V sub(V a, V b) { return make_double2(a.x - b.x, a.y - b.y); }
   static __device__ __forceinline__ V mul(V a, V b) { return make_double2(a.x * b.x, a.y * b.y); }
   static __device__ __forceinline__ V fma(V a, V b, V c) { return make_double2(::fma(a.x, b.x, c.x), ::fma(a.y, b.y, c.y)); }
-  static __device__ __forceinline__ V rcp(V a) { return make_double2(rcp_newton(a.x), rcp_newton(a.y)); }
+  static __device__ __forceinline__ V rcp(V a) { return make_double2(rcp_digits(a.x), rcp_digits(a.y)); }
 };
 
 // van Leer half-slopes of a pair: q = dl dr / (dl + dr) if dl dr > 0, else 0.
@@ -463,8 +442,17 @@ __device__ __forceinline__ typename P2<R>::V vl2(typename P2<R>::V x, typename P
   // both quotients are formed unconditionally and the select discards the
   // ones of non-positive products (including 0/0), so no branch is taken
   const auto q = P::mul(prod, P::rcp(s));                      // one (packed) multiply by reciprocals
-  return P::mk(pos_for_limiter(prod.x) ? q.x : R(0), pos_for_limiter(prod.y) ? q.y : R(0));
+  return P::mk(prod.x > R(0) ? q.x : R(0), prod.y > R(0) ? q.y : R(0));
 }
+template <>
+__device__ __forceinline__ double2 vl2<double>(double2 x, double2 y, double2 z) {
+  return make_double2(van_leer_digits(y.x - x.x, z.x - y.x), van_leer_digits(y.y - x.y, z.y - y.y));
+}
+// the same from the two differences
+__device__ __forceinline__ double2 vl2_of(double2 dl, double2 dr) {
+  return make_double2(van_leer_digits(dl.x, dr.x), van_leer_digits(dl.y, dr.y));
+}
+__device__ __forceinline__ float2 vl2_of(float2 dl, float2) { return dl; }      // FP32 forms its slopes with vl2
 
 template <typename R>
 __device__ __forceinline__ typename P2<R>::V sel2(bool cx, bool cy, typename P2<R>::V a, typename P2<R>::V b) {
