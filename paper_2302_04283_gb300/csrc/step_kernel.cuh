@@ -210,6 +210,37 @@ __device__ __forceinline__ double quartic_root(double B4, double B1, double B0, 
     f = fma(fma(B4, t2 * T, B1), T, B0);
     if (T > 0.0 && isfinite(T) && fabs(f) <= 1e-9 * -B0) return T;
   }
+  if (full64 && guess > 0.0) {
+    // FP32 iterations from the guess, then three FP64 Newton steps with the
+    // FP32 slope, each gaining six digits or more: 25 FP64 operations in place
+    // of several Newton steps with correctly rounded divisions (a cell's solve
+    // occupies the FP64 pipe like a whole warp's; in a 2D grid it runs per
+    // cell).  Kept if the last step is a rounding's size.
+    const float b4f = (float)B4, b1f = (float)B1, b0f = (float)B0;
+    float tf = fminf(-b0f / b1f, sqrtf(sqrtf(-b0f / b4f))), ifp = 0.0f;
+    {
+      const float g = (float)guess, g3 = g * g * g;
+      const float tg = g - __fdividef(fmaf(fmaf(b4f, g3, b1f), g, b0f), fmaf(4.0f * b4f, g3, b1f));
+      if (tg > 0.0f && tg < tf) tf = tg;
+    }
+    for (int it = 0; it < 40; ++it) {
+      const float t2 = tf * tf;
+      const float f = fmaf(fmaf(b4f, t2 * tf, b1f), tf, b0f);
+      ifp = __fdividef(1.0f, fmaf(4.0f * b4f, t2 * tf, b1f));
+      const float tn = tf - f * ifp;
+      if (!(tn < tf) || !(tn > 0.0f)) break;
+      tf = tn;
+    }
+    double T = (double)tf, d = 0.0;
+    const double sl = (double)ifp;
+#pragma unroll
+    for (int it = 0; it < 3; ++it) {
+      const double T2 = T * T;
+      d = fma(fma(B4, T2 * T, B1), T, B0) * sl;
+      T -= d;
+    }
+    if (T > 0.0 && fabs(d) <= 1e-15 * T) return T;
+  }
   // FP64: Newton from the upper bound decreases monotonically onto the root
   double T = fmin(-B0 / B1, sqrt(sqrt(-B0 / B4)));
   if (guess > 0.0) {
@@ -431,6 +462,11 @@ template <> struct P2<double> {
   static __device__ __forceinline__ V fma(V a, V b, V c) { return make_double2(::fma(a.x, b.x, c.x), ::fma(a.y, b.y, c.y)); }
   static __device__ __forceinline__ V rcp(V a) { return make_double2(rcp_digits(a.x), rcp_digits(a.y)); }
 };
+
+__device__ __forceinline__ bool exp_ones(float) { return false; }
+__device__ __forceinline__ bool exp_ones(double x) { return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000; }
+__device__ __forceinline__ float inv1(float x) { return 1.0f / x; }
+__device__ __forceinline__ double inv1(double x) { return rcp_digits(x); }
 
 // van Leer half-slopes of a pair: q = dl dr / (dl + dr) if dl dr > 0, else 0.
 template <typename R>
@@ -706,6 +742,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
       sgas[8 * c + 2] = uz;
       sgas[8 * c + 3] = (R)a.aa[cell] + (R)a.as[cell];
       sgas[8 * c + 4] = sqrt(R(1) + ux * ux + uy * uy + uz * uz);
+      if (sizeof(R) == 8) sgas[8 * c + 5] = sgas[8 * c + 3] * (R)a.dts;
     }
   }
   if (tau) {
@@ -766,7 +803,8 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
   const bool g0 = act0 && a.zero_guard && fabs((double)nlow0.x) < a.n0crit;
   const bool g1 = act1 && a.zero_guard && fabs((double)nlow0.y) < a.n0crit;
   // primitive recovery factor (0 for guarded or inactive bins)
-  const V inv_f = P::mk((act0 && !g0) ? R(1) / fconv.x : R(0), (act1 && !g1) ? R(1) / fconv.y : R(0));
+  const V inv_f = P::mk((act0 && !g0) ? inv1(fconv.x) : R(0), (act1 && !g1) ? inv1(fconv.y) : R(0));
+  const bool live0 = act0 && !g0, live1 = act1 && !g1;
   const V keep = P::mk((act0 && !g0) ? R(1) : R(0), (act1 && !g1) ? R(1) : R(0));   // 0: guarded or padding
   // The stage combination of U = n^0 n_0 I, U* = U^{s-1} + dt L (stage 1) or
   // (U^0 + U^1 + dt L) / 2 (stage 2) with L = -(divS + divA), taken back to
@@ -777,7 +815,14 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
   const V kS = P::mul(P::mk(hs, hs), keep);
   const V kD = P::mul(P::mk(-hs * (R)a.dt, -hs * (R)a.dt), inv_f);
   const R invdV = cg.invdV;
-  auto fcoef = [&](const Face &F, unsigned &upR) -> V {
+  auto fcoef = [&](int d, const Face &F, unsigned &upR) -> V {
+    if (sizeof(R) == 8 && !ANG) {
+      // Cartesian flat space: n^d is the direction's own component and n_0 = -1
+      const V nd = d == 0 ? nhx : (d == 1 ? nhy : nhz);
+      upR = (nd.x < R(0) ? 1u : 0u) | (nd.y < R(0) ? 2u : 0u);
+      const R f = F.m0[0] * F.dA * invdV;
+      return P::mk(act0 ? nd.x * f : R(0), act1 ? nd.y * f : R(0));
+    }
     V na = P::fma(nhz, P::mk(F.ea[3], F.ea[3]),
                   P::fma(nhy, P::mk(F.ea[2], F.ea[2]), P::fma(nhx, P::mk(F.ea[1], F.ea[1]), P::mk(F.ea[0], F.ea[0]))));
     V n0 = P::fma(nhz, P::mk(F.m0[3], F.m0[3]),
@@ -791,14 +836,14 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
   for (int d = 0; d < 3; ++d) cm[d] = cp[d] = P::mk(R(0), R(0));
   {
     const Face *F1 = (const Face *)a.f1, *F2 = (const Face *)a.f2, *F3 = (const Face *)a.f3;
-    cm[0] = fcoef(F1[j * (a.n1 + 1) + i], um[0]);
-    cp[0] = fcoef(F1[j * (a.n1 + 1) + i + 1], up[0]);
+    cm[0] = fcoef(0, F1[j * (a.n1 + 1) + i], um[0]);
+    cp[0] = fcoef(0, F1[j * (a.n1 + 1) + i + 1], up[0]);
     if (a.ndim >= 2) {
-      cm[1] = fcoef(F2[j * a.n1 + i], um[1]);
-      cp[1] = fcoef(F2[(j + 1) * a.n1 + i], up[1]);
+      cm[1] = fcoef(1, F2[j * a.n1 + i], um[1]);
+      cp[1] = fcoef(1, F2[(j + 1) * a.n1 + i], up[1]);
     }
     if (a.ndim >= 3) {
-      cm[2] = fcoef(F3[col], um[2]);
+      cm[2] = fcoef(2, F3[col], um[2]);
       cp[2] = cm[2];
       up[2] = um[2];
     }
@@ -829,16 +874,17 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
   // of the rows u2, u1, d1 in a ring stage.
   constexpr bool MIR = !ANG && !TAU && RC != RAD_RECON_PPM;
   const bool mir = MIR && (NAP != 0 || a.sign_pairs);
-  // In FP64 x3 takes the same form from the register window (its selects run
-  // on the integer pipe, beside the FP64 pipe that bounds that kernel); mXs
-  // is X with the sign of the mirror, which multiplies the own slope.
-  constexpr bool MIR3 = MIR && sizeof(R) == 8;
-  V mX[3], mY[3], mXs = P::mk(R(0), R(0));
-  bool dn3 = false;
+  // FP64 (FL64) takes this form along all three dimensions and on every flat
+  // grid (without sign pairs each bin selects its own side's rows), and folds
+  // the stage combination's factor kD into the coefficients: with P = kD X,
+  // Q = kD Y,  I* = kS I^0 [stage 2] + (kS + sum_d P_d) c
+  //                 + sum_d P_d q(u1, c, d1) + Q_d (u1 + q(u2, u1, c)).
+  constexpr bool FL64 = MIR && sizeof(R) == 8;
+  V mX[3], mY[3], pc = kS;
   int mo[2][3];
   if (MIR) {
 #pragma unroll
-    for (int d = 0; d < (MIR3 ? 3 : 2); ++d) {
+    for (int d = 0; d < (FL64 ? 3 : 2); ++d) {
       // the side of the element with the larger coefficient; a direction
       // component that is zero up to rounding (a few 1e-17: lattice points on
       // a coordinate plane) may carry either sign, and its flux is negligible
@@ -848,13 +894,16 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
       const bool dn = ax >= ay ? rx : ry;                // upwind on the upper side
       if (mir && rx != ry && fmin(ax, ay) > R(1e-6) * fmax(ax, ay)) atomicOr(a.err, kErrState);
       const V ncm = P::mk(-cm[d].x, -cm[d].y);
-      mX[d] = dn ? ncm : cp[d];
-      mY[d] = dn ? cp[d] : ncm;
-      if (d == 2) {
-        dn3 = dn;
-        mXs = dn ? P::mk(-mX[2].x, -mX[2].y) : mX[2];
-        continue;
+      const bool dx = FL64 && !mir ? rx : dn, dy = FL64 && !mir ? ry : dn;
+      mX[d] = P::mk(dx ? ncm.x : cp[d].x, dy ? ncm.y : cp[d].y);
+      mY[d] = P::mk(dx ? cp[d].x : ncm.x, dy ? cp[d].y : ncm.y);
+      if (FL64) {
+        mX[d] = P::mul(kD, mX[d]);
+        mY[d] = P::mul(kD, mY[d]);
+        pc = P::add(pc, mX[d]);
+        um[d] = (dx ? 1u : 0u) | (dy ? 2u : 0u);
       }
+      if (d == 2) continue;
       // x1: the block rows i-2 .. i+2 in slots 0 .. 4; x2: rows j-2, j-1,
       // j+1, j+2 in slots SX2 .. SX2 + 3
       const int s2 = d == 0 ? (dn ? 4 : 0) : SX2 + (dn ? 3 : 0);
@@ -866,6 +915,51 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
       mo[d][2] = sd * nap + bo;
     }
   }
+  // The FP64 kernels are bound by their pipe; per bin and stage this leaves 24
+  // operations of transport and 31 of coupling (54 and 48 before): 64^3 x 162
+  // with gas source 8.15 -> 6.43 ms per stage.
+  // FL64: acc + P q(u1, c, d1) + Q (u1 + q(u2, u1, c)) along x1 or x2
+  auto flux64 = [&](int d, const R *sr, V c, V acc) -> V {
+    V u1, u2 = c, d1 = c;
+    if (mir) {
+      u1 = *(const V *)(sr + mo[d][1]);
+      if (plm) {
+        u2 = *(const V *)(sr + mo[d][0]);
+        d1 = *(const V *)(sr + mo[d][2]);
+      }
+    } else {
+      const int bo = inpair ? b0 : 0;
+      const R *r = sr + (d == 0 ? 0 : SX2 * nap) + bo;         // rows at -2, -1, +1, +2
+      const int u = d == 0 ? 3 * nap : 2 * nap;
+      const V m1 = *(const V *)(r + nap), p1 = *(const V *)(r + u);
+      const bool dx = um[d] & 1, dy = um[d] & 2;
+      u1 = sel2<R>(dx, dy, p1, m1);
+      if (plm) {
+        const V m2 = *(const V *)r, p2 = *(const V *)(r + u + nap);
+        u2 = sel2<R>(dx, dy, p2, m2);
+        d1 = sel2<R>(dx, dy, m1, p1);
+      }
+    }
+    if (!plm) return P::fma(mY[d], u1, acc);
+    const V db = P::sub(c, u1);
+    const V qf = vl2_of(P::sub(u1, u2), db), qc = vl2_of(db, P::sub(d1, c));
+    return P::fma(mX[d], qc, P::fma(mY[d], P::add(u1, qf), acc));
+  };
+  // AN64 (curved space, FP64): the flux difference of one dimension from the
+  // two slopes its faces use, the faces' sides taken per bin
+  constexpr bool AN64 = ANG && !TAU && RC != RAD_RECON_PPM && sizeof(R) == 8;
+  auto div64 = [&](int d, V m2, V m1, V c, V p1, V p2, V sx) -> V {
+    const bool lx = um[d] & 1, ly = um[d] & 2, hx = up[d] & 1, hy = up[d] & 2;
+    V lo = sel2<R>(lx, ly, c, m1), hi = sel2<R>(hx, hy, p1, c);
+    if (plm) {
+      const V d0 = P::sub(m1, m2), d1 = P::sub(c, m1), d2 = P::sub(p1, c), d3 = P::sub(p2, p1);
+      const V ql = vl2_of(sel2<R>(lx, ly, d1, d0), sel2<R>(lx, ly, d2, d1));
+      const V qh = vl2_of(sel2<R>(hx, hy, d2, d1), sel2<R>(hx, hy, d3, d2));
+      lo = P::add(lo, P::mk(lx ? -ql.x : ql.x, ly ? -ql.y : ql.y));
+      hi = P::add(hi, P::mk(hx ? -qh.x : qh.x, hy ? -qh.y : qh.y));
+    }
+    return P::fma(cp[d], hi, P::fma(P::mk(-cm[d].x, -cm[d].y), lo, sx));
+  };
   auto divm = [&](int d, const R *sr, V c) -> V {
     const V u1 = *(const V *)(sr + mo[d][1]);
     if (!plm) return P::fma(mX[d], c, P::mul(mY[d], u1));
@@ -1075,7 +1169,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
   }
 
   // ---- phase A (consumer warps): transport, stage combination, primitive I*, coupling sums
-  V w0 = zero, w1 = zero, w2 = zero, w3 = zero, qa = zero, qb = zero;   // x3 window and slopes
+  V w0 = zero, w1 = zero, w2 = zero, w3 = zero, qa = zero, qb = zero, wd = zero;   // x3 window and slopes
   V pw[6];                                               // PPM x3 window, rows k-3 .. k+2
 #pragma unroll
   for (int q = 0; q < 6; ++q) pw[q] = zero;
@@ -1100,6 +1194,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
     if (plm) {
       qa = vl2<R>(w0, w1, w2);
       qb = vl2<R>(w1, w2, w3);
+      wd = P::sub(w3, w2);
     }
   }
   int st = 0;
@@ -1138,20 +1233,42 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
       sx = divs(2, loL, loR, hiL, hiR, dlo[2], dhi[2]);
 #pragma unroll
       for (int q = 0; q < 6; ++q) pw[q] = win[q + 1];
+    } else if (d3 && (FL64 || AN64)) {
+      // slopes: qa = slope(k-1), qb = slope(k), qc = slope(k+1); wd = w3 - w2
+      const V w4 = sv(sr + SX3 * nap), dr = P::sub(w4, w3);
+      const V qc = plm ? vl2_of(wd, dr) : zero;
+      zc = w2;
+      const bool dx = um[2] & 1, dy = um[2] & 2;         // the upwind side is k+1's
+      if (FL64) {
+        sx = P::fma(pc, zc, ST2 ? P::mul(kS, sv(sr + SI0 * nap)) : zero);
+        const V u1 = sel2<R>(dx, dy, w3, w1);
+        if (plm) {
+          sx = P::fma(mX[2], P::mk(dx ? -qb.x : qb.x, dy ? -qb.y : qb.y), sx);
+          sx = P::fma(mY[2], P::add(u1, P::mk(dx ? -qc.x : qa.x, dy ? -qc.y : qa.y)), sx);
+        } else {
+          sx = P::fma(mY[2], u1, sx);
+        }
+      } else {
+        V lo = sel2<R>(dx, dy, w2, w1), hi = sel2<R>(dx, dy, w3, w2);
+        if (plm) {
+          lo = P::add(lo, P::mk(dx ? -qb.x : qa.x, dy ? -qb.y : qa.y));
+          hi = P::add(hi, P::mk(dx ? -qc.x : qb.x, dy ? -qc.y : qb.y));
+        }
+        sx = P::mul(cm[2], P::sub(hi, lo));
+      }
+      w0 = w1;
+      w1 = w2;
+      w2 = w3;
+      w3 = w4;
+      wd = dr;
+      qa = qb;
+      qb = qc;
     } else if (d3) {
       const V w4 = sv(sr + SX3 * nap);
       const V qc = plm ? vl2<R>(w2, w3, w4) : zero;   // slope of k+1
       zc = w2;
       // slopes: qa = slope(k-1), qb = slope(k), qc = slope(k+1)
-      if (MIR3 && mir) {
-        // upwind frame: u1 = w1 or w3, its mirrored slope qa or -qc, the
-        // own mirrored slope +-qb (the sign in mXs)
-        const V u1 = dn3 ? w3 : w1;
-        sx = plm ? P::fma(mX[2], w2, P::fma(mXs, qb, P::mul(mY[2], P::add(u1, dn3 ? P::mk(-qc.x, -qc.y) : qa))))
-                 : P::fma(mX[2], w2, P::mul(mY[2], u1));
-      } else {
-        sx = divd(2, w1, w2, w3, qa, qb, qc, dlo[2], dhi[2]);
-      }
+      sx = divd(2, w1, w2, w3, qa, qb, qc, dlo[2], dhi[2]);
       w0 = w1;
       w1 = w2;
       w2 = w3;
@@ -1160,6 +1277,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
       qb = qc;
     } else {
       zc = sv(sr + H * nap);
+      if (FL64) sx = P::fma(pc, zc, ST2 ? P::mul(kS, sv(sr + SI0 * nap)) : zero);
     }
     if (ppm) {
       V v[7];
@@ -1168,6 +1286,10 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
       V loL, loR, hiL, hiR;
       ppm_states<R>(v, loL, loR, hiL, hiR);
       sx = P::add(sx, divs(0, loL, loR, hiL, hiR, dlo[0], dhi[0]));
+    } else if (FL64) {
+      sx = flux64(0, sr, zc, sx);
+    } else if (AN64) {
+      sx = div64(0, sv(sr), sv(sr + nap), zc, sv(sr + 3 * nap), sv(sr + 4 * nap), sx);
     } else if (mir) {
       sx = P::add(sx, divm(0, sr, zc));
     } else {
@@ -1191,6 +1313,8 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
       V loL, loR, hiL, hiR;
       ppm_states<R>(v, loL, loR, hiL, hiR);
       sx = P::add(sx, divs(1, loL, loR, hiL, hiR, dlo[1], dhi[1]));
+    } else if (a.ndim >= 2 && FL64) {
+      sx = flux64(1, sr, zc, sx);
     } else if (a.ndim >= 2 && mir) {
       sx = P::add(sx, divm(1, sr, zc));
     } else if (a.ndim >= 2) {
@@ -1200,6 +1324,9 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
         const R *row = sr + (SX2 + q) * nap;
         yv[q] = (ANG && anypol && ypol[q] == 1) ? P::mk(row[p0], row[p1]) : sv(row);
       }
+      if (AN64) {
+        sx = div64(1, yv[0], yv[1], zc, yv[2], yv[3], sx);
+      } else {
       V sm = zero, sc = zero, sp = zero;
       if (plm) {
         sm = vl2<R>(yv[0], yv[1], zc);
@@ -1207,6 +1334,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
         sp = vl2<R>(zc, yv[2], yv[3]);
       }
       sx = P::add(sx, divd(1, yv[1], zc, yv[2], sm, sc, sp, dlo[1], dhi[1]));
+      }
     }
     V divA = zero;
     if (ANG && AM) {
@@ -1293,12 +1421,16 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
     }
     // U* = U^{s-1} + dt L   (stage 1)   or   U^0/2 + (U^1 + dt L)/2   (stage 2), L = -(divS + divA)
     if (ANG) sx = P::add(sx, divA);
-    if (EXT && a.divF) sx = P::add(sx, __ldg((const V *)((const R *)a.divF + (unsigned)(k0 + c) * strideK + own)));
+    if (EXT && a.divF && FL64)
+      sx = P::fma(kD, __ldg((const V *)((const R *)a.divF + (unsigned)(k0 + c) * strideK + own)), sx);
+    else if (EXT && a.divF) sx = P::add(sx, __ldg((const V *)((const R *)a.divF + (unsigned)(k0 + c) * strideK + own)));
     // FP64: the affine form (fewer FP64-pipe operations); FP32: U* first and
     // I* after the release (the FP32 kernels' register allocation prefers it)
     constexpr bool AFF = sizeof(R) == 8;
     V Is = zero, Us = zero;
-    if (AFF) {
+    if (FL64) {
+      Is = sx;
+    } else if (AFF) {
       Is = ST2 ? P::fma(kS, P::add(sv(sr + SI0 * nap), zc), P::mul(kD, sx)) : P::fma(kS, zc, P::mul(kD, sx));
     } else {
       Us = P::fma(P::mk(-dtR, -dtR), sx, P::mul(fconv, zc));   // L = -(divS + divA)
@@ -1318,7 +1450,19 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
     if (!AFF) Is = P::mul(Us, inv_f);
     if (inpair) *(V *)(sI + c * nap + b0) = Is;
     if (a.Istar && inpair) *(V *)((R *)a.Istar + (unsigned)(k0 + c) * strideK + own) = Is;
-    if (couple) {
+    if (couple && sizeof(R) == 8) {
+      // FP64, in the fewest operations of its pipe: r2 = 1 / (n^0bar den),
+      // t = n^0bar^2 r2 = n^0bar / den; the factor -alpha_E dt of
+      // (c1 - 1) = -alpha_E dt t is common to the bins and applied in phase B
+      const GasRow<R> grow = gas_load(sgas + 8 * c);
+      const R *g = grow.v;
+      const V nb = P::fma(P::mk(-g[0], -g[0]), nhx, P::fma(P::mk(-g[1], -g[1]), nhy,
+                                                           P::fma(P::mk(-g[2], -g[2]), nhz, P::mk(g[4], g[4]))));
+      const V r2 = P::rcp(P::mul(nb, P::fma(nb, P::mk(g[5], g[5]), P::mk(n0up, n0up))));
+      const V nb2 = P::mul(nb, nb), w = P::mul(Is, P::mul(nb2, dOm)), t2 = P::mul(nb2, r2);
+      const R s2 = warp_reduce4<R>(t2.x * w.x + t2.y * w.y, dOm.x * r2.x + dOm.y * r2.y, w.x + w.y, R(0), lane);
+      if ((lane & 7) == 0 && lane < 24) red[(c * nwarp + warp) * kNRedC + (lane >> 3)] = s2;
+    } else if (couple) {
       const GasRow<R> grow = gas_load(sgas + 8 * c);
       const R *g = grow.v;
       const V ux = P::mk(g[0], g[0]), uy = P::mk(g[1], g[1]), uz = P::mk(g[2], g[2]);
@@ -1359,7 +1503,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
       for (int w = 0; w < nwarp; ++w)
 #pragma unroll
         for (int r = 0; r < kNRedA; ++r) rs[r] += red[(c * nwarp + w) * kNRedC + r];
-      const double D = (double)rs[0], A2 = a.dts / kFourPi * (double)rs[1], Em = (double)rs[2];
+      const double D = sizeof(R) == 8 ? -(double)(sgas[8 * c + 5] * rs[0]) : (double)rs[0], A2 = a.dts / kFourPi * (double)rs[1], Em = (double)rs[2];
       double S, Tp = Tst;
       bool ok = true;
       if (a.mode == RAD_COUPLE_THERMAL) {
@@ -1379,7 +1523,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
         S = kFourPi * eta + as * Ep;
       }
       if (!ok || !isfinite(Tp) || !isfinite(S)) atomicOr(a.err, kErrNoConv);
-      Sc[c] = (R)S;
+      Sc[c] = sizeof(R) == 8 ? c2pre * (R)S : (R)S;      // FP64: with the bins' common factor
       a.Tout[cell] = Tp;
     }
     __syncthreads();
@@ -1401,7 +1545,16 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
   auto implicit = [&](int c, V &Is, V &out) {
     Is = inpair ? *(const V *)(sI + c * nap + b0) : zero;
     out = Is;
-    if (couple) {
+    if (couple && sizeof(R) == 8) {
+      const GasRow<R> grow = gas_load(sgas + 8 * c);
+      const R *g = grow.v;
+      const V nb = P::fma(P::mk(-g[0], -g[0]), nhx, P::fma(P::mk(-g[1], -g[1]), nhy,
+                                                           P::fma(P::mk(-g[2], -g[2]), nhz, P::mk(g[4], g[4]))));
+      const V nb3 = P::mul(nb, P::mul(nb, nb));
+      const V q = P::rcp(P::mul(nb3, P::fma(nb, P::mk(g[5], g[5]), P::mk(n0up, n0up))));
+      const V c1 = P::mul(ANG ? P::mul(P::mk(n0up, n0up), nb3) : nb3, q);      // n^0 = 1 in Cartesian space
+      out = P::fma(c1, Is, P::mul(q, P::mk(Sc[c], Sc[c])));
+    } else if (couple) {
       const GasRow<R> grow = gas_load(sgas + 8 * c);
       const R *g = grow.v;
       const V ux = P::mk(g[0], g[0]), uy = P::mk(g[1], g[1]), uz = P::mk(g[2], g[2]);
@@ -1417,13 +1570,29 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
   // gas source: the pair's share of sum (I+ - I*) n^A dOmega (before the guard)
   auto src4 = [&](V Is, V out, R (&v)[4]) {
     const V d = P::mul(P::sub(out, Is), dOm);
+    if (sizeof(R) == 8) {
+      v[0] = d.x + d.y;
+      v[1] = d.x * nhx.x + d.y * nhx.y;
+      v[2] = d.x * nhy.x + d.y * nhy.y;
+      v[3] = d.x * nhz.x + d.y * nhz.y;
+      return;
+    }
     const V dx = P::mul(d, nhx), dy = P::mul(d, nhy), dz = P::mul(d, nhz);
     v[0] = d.x + d.y;
     v[1] = dx.x + dx.y;
     v[2] = dy.x + dy.y;
     v[3] = dz.x + dz.y;
   };
+  bool nonfin = false;    // FP64: an exponent of all ones, on the integer pipe
   auto store = [&](int c, V out) {
+    if (sizeof(R) == 8) {
+      out = sel2<R>(live0, live1, out, zero);
+      if (inpair) {
+        *(V *)(Io + (unsigned)(k0 + c) * strideK + own) = out;
+        nonfin |= exp_ones(out.x) || exp_ones(out.y);
+      }
+      return;
+    }
     out = P::mul(out, keep);
     if (inpair) {
       *(V *)(Io + (unsigned)(k0 + c) * strideK + own) = out;
@@ -1507,7 +1676,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
     }
     store(c, out);
   }
-  const bool bad = !isfinite(chk.x) || !isfinite(chk.y);
+  const bool bad = sizeof(R) == 8 ? nonfin : !isfinite(chk.x) || !isfinite(chk.y);
   if (cons && __any_sync(0xffffffffu, bad) && lane == 0) atomicOr(a.err, kErrNonFinite);
   if (want_src) {
     // ---- phase D: -dR^0_mu with dR^0_mu = n^0 M[mu][A] sum (I+ - I*) n^A dOmega
