@@ -91,6 +91,7 @@ void rad_destroy(rad_ctx *ctx) {
   }
   cudaFree(ctx->host_slot_buf);
   cudaFree(ctx->nu_edges_dev);
+  cudaFree(ctx->grp_tab);
   cudaFree(ctx->freq_buf);
   delete ctx;
 }
@@ -467,12 +468,24 @@ int rad_set_groups(rad_ctx *ctx, int n_groups, const double *nu_edges) {
   if (n_groups > 0 && !(nu_edges[0] >= 0.0)) return fail(ctx, RAD_EINVAL, "the lowest edge must be >= 0");
   cudaStreamSynchronize(ctx->stream);
   cudaFree(ctx->nu_edges_dev);
+  cudaFree(ctx->grp_tab);
+  ctx->grp_tab = nullptr;
   ctx->nu_edges_dev = nullptr;
   ctx->nu_edges.clear();
   ctx->n_groups = 0;
   if (n_groups == 0) return RAD_OK;
   ctx->nu_edges.assign(nu_edges, nu_edges + n_groups + 1);
   cudaError_t ce = upload(&ctx->nu_edges_dev, ctx->nu_edges, ctx->stream);
+  // the frequency flux kernel's table: an edge at 0 or infinity carries
+  // nothing (0 here), a group reaching infinity has infinite width
+  const int nt = 2 * n_groups + 1;
+  std::vector<double> tab(nt + (nt + 1) / 2, 0.0);
+  std::vector<float> tabf(nt, 0.0f);
+  for (int f = 0; f <= n_groups; ++f) tab[f] = std::isinf(nu_edges[f]) ? 0.0 : nu_edges[f];
+  for (int g = 0; g < n_groups; ++g) tab[n_groups + 1 + g] = nu_edges[g + 1] - nu_edges[g];
+  for (int q = 0; q < nt; ++q) tabf[q] = (float)tab[q];
+  std::memcpy(tab.data() + nt, tabf.data(), nt * sizeof(float));
+  if (ce == cudaSuccess) ce = upload(&ctx->grp_tab, tab, ctx->stream);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(ctx->stream);
   if (ce != cudaSuccess) return fail(ctx, RAD_ENOMEM, std::string("group edge upload failed: ") + cudaGetErrorString(ce));
   ctx->n_groups = n_groups;

@@ -151,6 +151,7 @@ struct rad_ctx {
   int n_groups = 0;
   std::vector<double> nu_edges;
   double *nu_edges_dev = nullptr;
+  double *grp_tab = nullptr;    // edge frequencies [n_groups + 1] and widths [n_groups], FP64 then FP32 (frequency.cu)
   void *freq_buf = nullptr;
   size_t freq_bytes = 0;
   // rad_step_adjoint scratch

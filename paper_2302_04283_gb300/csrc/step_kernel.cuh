@@ -91,7 +91,11 @@ struct StageArgs {
   double tau_const;       // C of the optical-depth flux weighting (0: free streaming)
   int *err;
   const void *halo[6];     // ghost rows of faces shared with other blocks: face (d, side) at 2 d + side
-  const void *divF;        // multigroup: this group's frequency divergence [cell][nap] (null: gray)
+  const void *divF;        // multigroup: the groups' frequency divergence [group][cell][nap] (null: gray)
+  // multigroup: all groups in one launch, blockIdx.y the group; its intensity
+  // arrays, opacities, emissivity and source start gI elements / gC cells on
+  int ngrp;
+  size_t gI, gC;
 };
 
 StageArgs make_stage_args(rad_ctx *ctx, const rad_gas *gas, double dt, const rad_opts *o, double *gas_src);
@@ -714,6 +718,20 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
   const R *Ip = (const R *)a.Iprev;
   const R *I0 = (const R *)a.I0;
   R *Io = (R *)a.Iout;
+  const double *gaa = a.aa, *gas_ = a.as, *geta = a.eta;
+  double *gsrc = a.src;
+  const R *gdiv = (const R *)a.divF;
+  if (EXT && a.ngrp > 1) {               // this CTA's frequency group
+    const size_t oI = blockIdx.y * a.gI, oC = blockIdx.y * a.gC;
+    Ip += oI;
+    I0 += oI;
+    Io += oI;
+    gdiv += oI;
+    if (gaa) gaa += oC;
+    if (gas_) gas_ += oC;
+    if (geta) geta += oC;
+    if (gsrc) gsrc += 4 * oC;
+  }
   constexpr bool plm = RC == RAD_RECON_PLM;
   constexpr bool ppm = RC == RAD_RECON_PPM;
   constexpr int H = ppm ? 3 : 2;                           // stencil half-width
@@ -740,7 +758,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
       sgas[8 * c + 0] = ux;
       sgas[8 * c + 1] = uy;
       sgas[8 * c + 2] = uz;
-      sgas[8 * c + 3] = (R)a.aa[cell] + (R)a.as[cell];
+      sgas[8 * c + 3] = (R)gaa[cell] + (R)gas_[cell];
       sgas[8 * c + 4] = sqrt(R(1) + ux * ux + uy * uy + uz * uz);
       if (sizeof(R) == 8) sgas[8 * c + 5] = sgas[8 * c + 3] * (R)a.dts;
     }
@@ -770,7 +788,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
       const unsigned nbc = (unsigned)kk * ncol + (unsigned)jj * a.n1 + ii;
       const R uxo = (R)a.u[3 * cell], uyo = (R)a.u[3 * cell + 1], uzo = (R)a.u[3 * cell + 2];
       const R uxn = (R)a.u[3 * nbc], uyn = (R)a.u[3 * nbc + 1], uzn = (R)a.u[3 * nbc + 2];
-      const R aEo = (R)a.aa[cell] + (R)a.as[cell], aEn = (R)a.aa[nbc] + (R)a.as[nbc];
+      const R aEo = (R)gaa[cell] + (R)gas_[cell], aEn = (R)gaa[nbc] + (R)gas_[nbc];
       const R fx = R(0.5) * (uxo + uxn), fy = R(0.5) * (uyo + uyn), fz = R(0.5) * (uzo + uzn);
       const R u0F = sqrt(R(1) + fx * fx + fy * fy + fz * fz);
       const R tq = (R)a.tau_const * (R(0.5) * (aEo + aEn)) * (R)a.dt / u0F;
@@ -1421,9 +1439,9 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
     }
     // U* = U^{s-1} + dt L   (stage 1)   or   U^0/2 + (U^1 + dt L)/2   (stage 2), L = -(divS + divA)
     if (ANG) sx = P::add(sx, divA);
-    if (EXT && a.divF && FL64)
-      sx = P::fma(kD, __ldg((const V *)((const R *)a.divF + (unsigned)(k0 + c) * strideK + own)), sx);
-    else if (EXT && a.divF) sx = P::add(sx, __ldg((const V *)((const R *)a.divF + (unsigned)(k0 + c) * strideK + own)));
+    if (EXT && gdiv && FL64)
+      sx = P::fma(kD, __ldg((const V *)(gdiv + (unsigned)(k0 + c) * strideK + own)), sx);
+    else if (EXT && gdiv) sx = P::add(sx, __ldg((const V *)(gdiv + (unsigned)(k0 + c) * strideK + own)));
     // FP64: the affine form (fewer FP64-pipe operations); FP32: U* first and
     // I* after the release (the FP32 kernels' register allocation prefers it)
     constexpr bool AFF = sizeof(R) == 8;
@@ -1493,12 +1511,12 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
     if (t < nc) {
       const int c = t, k = k0 + c;
       const unsigned cell = (unsigned)k * ncol + col;
-      if (ST2 && a.src) {                  // stage 1's share of the source, added to in phase D
+      if (ST2 && gsrc) {                  // stage 1's share of the source, added to in phase D
 #pragma unroll
-        for (int m = 0; m < 4; ++m) psrc[m] = a.src[4 * cell + m];
+        for (int m = 0; m < 4; ++m) psrc[m] = gsrc[4 * cell + m];
       }
       const double Tst = ST2 ? 0.5 * (a.T0[cell] + a.T1[cell]) : a.T0[cell];
-      const double aa = a.aa[cell], as = a.as[cell];
+      const double aa = gaa[cell], as = gas_[cell];
       R rs[kNRedA] = {R(0), R(0), R(0)};
       for (int w = 0; w < nwarp; ++w)
 #pragma unroll
@@ -1516,7 +1534,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
         const double T2 = Tp * Tp;
         S = aa * a.a_rad * T2 * T2 + as * Ep;
       } else {
-        const double eta = a.eta[cell];
+        const double eta = geta[cell];
         const double den = 1.0 - A2 * as;
         ok = den > 0.0;
         const double Ep = (D + Em + kFourPi * A2 * eta) / den;
@@ -1532,15 +1550,15 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
     if (t < nc) {
       const unsigned cell = (unsigned)(k0 + t) * ncol + col;
       a.Tout[cell] = ST2 ? 0.5 * (a.T0[cell] + a.T1[cell]) : a.T0[cell];
-      if (a.src && !ST2) {
-        for (int m = 0; m < 4; ++m) a.src[4 * cell + m] = 0.0;
+      if (gsrc && !ST2) {
+        for (int m = 0; m < 4; ++m) gsrc[4 * cell + m] = 0.0;
       }
     }
   }
 
   // ---- phase C: implicit update of every bin
   V chk = zero;           // stays 0 unless a written value is not finite (0 * inf, 0 * nan = nan)
-  const bool want_src = couple && a.src;
+  const bool want_src = couple && gsrc;
   // I+ of one cell before the guard, from I* and the cell's source S
   auto implicit = [&](int c, V &Is, V &out) {
     Is = inpair ? *(const V *)(sI + c * nap + b0) : zero;
@@ -1691,7 +1709,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
         for (int w = 0; w < nwarp; ++w) s += red[(c * nwarp + w) * kNRedC + A];
         xs[A] = s;
       }
-      double *sp = a.src + 4 * cell;
+      double *sp = gsrc + 4 * cell;
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
         R dR = n0up * (cg.M[m][0] * xs[0] + cg.M[m][1] * xs[1] + cg.M[m][2] * xs[2] + cg.M[m][3] * xs[3]);
