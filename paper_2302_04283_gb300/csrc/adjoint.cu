@@ -187,27 +187,31 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
     if (sizeof(W) == 8) g[4] *= dts;
   }
   __syncthreads();
-  // per bin and cell: nb = n^0bar, rden = 1 / (n^0 + nb alpha_E dt),
-  // c2n = c2pre rden / nb^3, wb = nb^2 dOmega, rn = dOmega rden / nb.  FP64
-  // takes all quotients from one reciprocal of nb den.
-  struct Bin { W nb, rden, c2n, wb, rn, inb; };
+  constexpr bool D64 = sizeof(W) == 8;
+  // per bin and cell: nb = n^0bar, rden = 1 / (n^0 + nb alpha_E dt), wb = nb^2
+  // dOmega.  FP64: r = 1 / (nb den) gives rden = nb r and inb = 1 / nb = den r;
+  // factors common to a cell's bins (alpha_E dt, dt, dt / 4 pi, n^0, S) are
+  // taken out of the sums, to save operations of the FP64 pipe.  FP32: c2n =
+  // c2pre rden / nb^3 and rn = dOmega rden / nb.
+  struct Bin { W nb, rden, wb, r, inb, c2n, rn; };
   auto bin = [&](int c) -> Bin {
     const W *g = gas + 8 * c;
     Bin b;
-    b.nb = g[3] - (g[0] * x + g[1] * y + g[2] * z);
-    b.wb = b.nb * b.nb * dOm;
-    if (sizeof(W) == 8) {
-      const W den = n0up + b.nb * g[4];
-      const W r = P2<W>::rcp(P2<W>::mk(b.nb * den, W(1))).x;
-      b.rden = b.nb * r;
-      b.inb = den * r;
-      b.c2n = c2p * b.rden * (b.inb * b.inb * b.inb);
-      b.rn = dOm * r;
+    if (D64) {
+      b.nb = fma_rn(-g[0], x, fma_rn(-g[1], y, fma_rn(-g[2], z, g[3])));
+      const W den = fma_rn(b.nb, g[4], n0up);
+      b.r = inv1(b.nb * den);
+      b.rden = b.nb * b.r;
+      b.inb = den * b.r;
+      b.wb = b.nb * b.nb * dOm;
+      b.c2n = b.rn = W(0);
     } else {
+      b.nb = g[3] - (g[0] * x + g[1] * y + g[2] * z);
+      b.wb = b.nb * b.nb * dOm;
       b.rden = W(1) / (n0up + b.nb * g[4] * dts);
       b.c2n = c2p * b.rden / (b.nb * b.nb * b.nb);
       b.rn = dOm * b.rden / b.nb;
-      b.inb = W(0);
+      b.r = b.inb = W(0);
     }
     return b;
   };
@@ -219,9 +223,10 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
     const W lp = live ? (W)lam[own + c * strideK] : W(0);
     const Bin b = bin(c);
     W s;
-    if (THERMAL) {
-      const W w = Is * b.wb;
-      s = warp_reduce4(-(b.nb * gas[8 * c + 4]) * b.rden * w, b.rn, w, b.c2n * lp, lane);
+    if (D64) {
+      const W w = Is * b.wb, v3 = b.rden * b.inb * (b.inb * b.inb) * lp;
+      s = THERMAL ? warp_reduce4(b.nb * b.rden * w, dOm * b.r, w, v3, lane)
+                  : warp_reduce4(b.rden * w, dOm * b.r, v3, W(0), lane);
     } else {
       const W c1 = n0up * b.rden;
       s = warp_reduce4(act ? c1 * Is * b.wb : W(0), act ? b.rn : W(0), act ? b.c2n * lp : W(0), W(0), lane);
@@ -237,6 +242,10 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
 #pragma unroll
       for (int r = 0; r < 4; ++r) t[r] += red[(c * nwarp + w) * 4 + r];
     W *o = sc + 8 * c;
+    if (D64) {                              // the common factors of the sums
+      t[0] *= THERMAL ? -gas[8 * c + 4] : n0up;
+      t[THERMAL ? 3 : 2] *= c2p;
+    }
     const W A2 = c2p * t[1], lS = THERMAL ? t[3] : t[2];
     if (THERMAL) {
       // the quartic B4 T^4 + B1 T + B0 = 0, Ebar+ = Ebar- - c_v (T+ - T-),
@@ -271,7 +280,7 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
       lA2 += -cv * asd * lB1 + aad * ar * lB4;
       las -= cv * A2 * lB1;
       laa += A2 * ar * lB4;
-      o[0] = aad * ar * T4 + asd * Ep;       // S
+      o[0] = c2p * (aad * ar * T4 + asd * Ep);   // c2pre S
       o[1] = lB0;                            // lambda_D
       o[2] = lEm;
       o[3] = c2p * lA2;                      // lambda of sum dOmega rden / n^0bar
@@ -290,9 +299,9 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
       const W lA2 = W(kFourPi) * eta * lEp / Q - as * lQ;
       const W leta = W(kFourPi) * lS + W(kFourPi) * A2 * lEp / Q;
       const W las = Ep * lS - A2 * lQ;
-      o[0] = S;
+      o[0] = D64 ? c2p * S : S;
       o[1] = lA1;
-      o[3] = lA2;
+      o[3] = D64 ? c2p * lA2 : lA2;
       o[4] = W(0);
       o[5] = las;
       if (A.g_eta) A.g_eta[cell] += (double)leta;
@@ -309,24 +318,21 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
     const W lp = live ? (W)lam[e] : W(0);
     const Bin b = bin(c);
     const W *o = sc + 8 * c;
-    const W S = o[0], lD = o[1];
-    const W c1 = n0up * b.rden;
-    W lIs, vE, lrden = W(0), cm1 = W(0);
-    const W lEm = THERMAL ? o[2] : W(0), lA2 = o[3];
-    if (THERMAL) {
-      cm1 = -(b.nb * gas[8 * c + 4]) * b.rden;
-      const W lc1 = Is * (lp + b.wb * lD);
-      lIs = c1 * lp + b.wb * (cm1 * lD + lEm);
-      lrden = n0up * lc1 + c2p * (b.inb * b.inb * b.inb) * (S * lp) + dOm * b.inb * lA2;
-      vE = -b.nb * dts * b.rden * b.rden * lrden;
+    const W S = o[0], lD = o[1], lA2 = o[3];
+    const W lEm = THERMAL ? o[2] : W(0);
+    W lIs, vE, lrden = W(0);
+    if (D64) {
+      // lambda of rden = 1 / den; vE without its factor -dt
+      const W wl = b.wb * lD, h = lp + wl;
+      lrden = fma_rn(n0up * Is, h, fma_rn(S, b.inb * b.inb * b.inb * lp, dOm * b.inb * lA2));
+      vE = b.rden * b.rden * b.nb * lrden;
+      lIs = THERMAL ? fma_rn(b.rden, fma_rn(-(b.nb * gas[8 * c + 4]), wl, n0up * lp), b.wb * lEm) : n0up * b.rden * h;
     } else {
+      const W c1 = n0up * b.rden;
       const W lc1 = Is * lp + Is * b.wb * lD;
       const W lc2n = S * lp;
       lIs = c1 * lp + c1 * b.wb * lD;
-      // FP64: dOmega rden^2 / nb as rn rden, without another quotient
-      const W lden = sizeof(W) == 8
-                         ? -c1 * b.rden * lc1 - b.c2n * b.rden * lc2n - c2p * b.rn * b.rden * lA2
-                         : -c1 * b.rden * lc1 - b.c2n * b.rden * lc2n - c2p * dOm * b.rden * b.rden / b.nb * lA2;
+      const W lden = -c1 * b.rden * lc1 - b.c2n * b.rden * lc2n - c2p * dOm * b.rden * b.rden / b.nb * lA2;
       vE = b.nb * dts * lden;
     }
     if (!act) vE = W(0);
@@ -337,8 +343,9 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
       W du[3] = {W(0), W(0), W(0)};
       if (act) {
         const W *g = gas + 8 * c;
-        const W dLdnb = -lrden * g[4] * b.rden * b.rden - W(3) * b.c2n * b.inb * S * lp +
-                        (cm1 * Is * lD + Is * lEm) * W(2) * b.nb * dOm - lA2 * b.rn * b.inb;
+        const W cm1 = -(b.nb * g[4]) * b.rden;
+        const W dLdnb = -lrden * g[4] * b.rden * b.rden - W(3) * b.rden * (b.inb * b.inb) * (b.inb * b.inb) * S * lp +
+                        (cm1 * Is * lD + Is * lEm) * W(2) * b.nb * dOm - lA2 * dOm * b.r * b.inb;
         const W iu0 = W(1) / g[3];
         du[0] = dLdnb * (g[0] * iu0 - x);
         du[1] = dLdnb * (g[1] * iu0 - y);
@@ -370,6 +377,7 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
     W t[4] = {W(0), W(0), W(0), W(0)};
     for (int w = 0; w < nwarp; ++w)
       for (int r = 0; r < nr; ++r) t[r] += red[(c * nwarp + w) * 4 + r];
+    if (D64) t[0] *= -dts;
     const W *o = sc + 8 * c;
     A.g_aa[cell] += THERMAL ? (double)(o[4] + t[0]) : (double)t[0];
     A.g_as[cell] += (double)(t[0] + o[5]);
