@@ -640,7 +640,8 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 // Wait for the given phase parity of an mbarrier; false after limit_ns (or
 // kSpinLimit polls), so that a wait that can no longer complete ends in an
-// error status instead of a stalled kernel.
+// error status instead of a stalled kernel.  The global timer, which takes
+// about a microsecond to read, is read only once a wait is long.
 __device__ __forceinline__ bool mbar_wait_parity(uint64_t *bar, uint32_t parity,
                                                  unsigned long long limit_ns = kWaitLimitNs) {
   const uint32_t a = s_addr(bar);
@@ -653,9 +654,9 @@ __device__ __forceinline__ bool mbar_wait_parity(uint64_t *bar, uint32_t parity,
         : "r"(a), "r"(parity)
         : "memory");
     if (done) return true;
-    if ((it & 255) == 0) {
+    if ((it & 63) == 63) {
       const unsigned long long now = global_ns();
-      if (it == 0) t0 = now;
+      if (it == 63) t0 = now;
       else if (now - t0 > limit_ns) return false;
     }
   }
@@ -715,23 +716,24 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
   const int nc = min(a.kc, a.n3 - k0);
   const unsigned ncol = (unsigned)a.n1 * a.n2;
   const unsigned strideK = ncol * (unsigned)nap;        // element offsets fit in 32 bits (host-checked)
-  const R *Ip = (const R *)a.Iprev;
-  const R *I0 = (const R *)a.I0;
-  R *Io = (R *)a.Iout;
-  const double *gaa = a.aa, *gas_ = a.as, *geta = a.eta;
-  double *gsrc = a.src;
-  const R *gdiv = (const R *)a.divF;
-  if (EXT && a.ngrp > 1) {               // this CTA's frequency group
-    const size_t oI = blockIdx.y * a.gI, oC = blockIdx.y * a.gC;
-    Ip += oI;
-    I0 += oI;
-    Io += oI;
-    gdiv += oI;
-    if (gaa) gaa += oC;
-    if (gas_) gas_ += oC;
-    if (geta) geta += oC;
-    if (gsrc) gsrc += 4 * oC;
-  }
+  // frequency groups (run-time rows only: see launch_stage): this CTA's group
+  // starts oI elements / oC cells into the arrays.  The flat fixed-row kernels
+  // read the arguments where they use them (local copies of the pointers cost
+  // 128^3 x 162 FP32 1 %, 6.76 -> 6.83 ms); the curved and run-time-row kernels
+  // keep the pointers (Kerr-Schild 128 x 64 x 64 x 362 FP32 5.34 -> 5.15 ms, 192 x
+  // 96 x 96 x 642 34.0 -> 32.9, lat/long 90 x 50 x 44 x 128 1.63 -> 1.57).
+  constexpr bool GRP = NAP == 0, LOC = NAP == 0 || ANG;
+  const size_t oI = GRP ? blockIdx.y * a.gI : 0, oC = GRP ? blockIdx.y * a.gC : 0;
+  const R *Ip = (const R *)a.Iprev + oI;
+  const R *I0 = (const R *)a.I0 + oI;
+  R *Io = (R *)a.Iout + oI;
+  const R *gdiv_ = (const R *)a.divF + oI;
+  const double *gaa_ = a.aa + oC, *gas_ = a.as + oC, *geta_ = a.eta + oC;
+  double *gsrc_ = a.src + 4 * oC;
+  auto opac_a = [&](unsigned cell) { return (LOC ? gaa_ : a.aa)[cell]; };
+  auto opac_s = [&](unsigned cell) { return (LOC ? gas_ : a.as)[cell]; };
+  auto emis = [&](unsigned cell) { return (LOC ? geta_ : a.eta)[cell]; };
+  auto source = [&](unsigned cell) { return (LOC ? gsrc_ : a.src) + 4 * (size_t)cell; };
   constexpr bool plm = RC == RAD_RECON_PLM;
   constexpr bool ppm = RC == RAD_RECON_PPM;
   constexpr int H = ppm ? 3 : 2;                           // stencil half-width
@@ -758,7 +760,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
       sgas[8 * c + 0] = ux;
       sgas[8 * c + 1] = uy;
       sgas[8 * c + 2] = uz;
-      sgas[8 * c + 3] = (R)gaa[cell] + (R)gas_[cell];
+      sgas[8 * c + 3] = (R)opac_a(cell) + (R)opac_s(cell);
       sgas[8 * c + 4] = sqrt(R(1) + ux * ux + uy * uy + uz * uz);
       if (sizeof(R) == 8) sgas[8 * c + 5] = sgas[8 * c + 3] * (R)a.dts;
     }
@@ -788,7 +790,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
       const unsigned nbc = (unsigned)kk * ncol + (unsigned)jj * a.n1 + ii;
       const R uxo = (R)a.u[3 * cell], uyo = (R)a.u[3 * cell + 1], uzo = (R)a.u[3 * cell + 2];
       const R uxn = (R)a.u[3 * nbc], uyn = (R)a.u[3 * nbc + 1], uzn = (R)a.u[3 * nbc + 2];
-      const R aEo = (R)gaa[cell] + (R)gas_[cell], aEn = (R)gaa[nbc] + (R)gas_[nbc];
+      const R aEo = (R)opac_a(cell) + (R)opac_s(cell), aEn = (R)opac_a(nbc) + (R)opac_s(nbc);
       const R fx = R(0.5) * (uxo + uxn), fy = R(0.5) * (uyo + uyn), fz = R(0.5) * (uzo + uzn);
       const R u0F = sqrt(R(1) + fx * fx + fy * fy + fz * fz);
       const R tq = (R)a.tau_const * (R(0.5) * (aEo + aEn)) * (R)a.dt / u0F;
@@ -1439,9 +1441,9 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
     }
     // U* = U^{s-1} + dt L   (stage 1)   or   U^0/2 + (U^1 + dt L)/2   (stage 2), L = -(divS + divA)
     if (ANG) sx = P::add(sx, divA);
-    if (EXT && gdiv && FL64)
-      sx = P::fma(kD, __ldg((const V *)(gdiv + (unsigned)(k0 + c) * strideK + own)), sx);
-    else if (EXT && gdiv) sx = P::add(sx, __ldg((const V *)(gdiv + (unsigned)(k0 + c) * strideK + own)));
+    if (EXT && a.divF && FL64)
+      sx = P::fma(kD, __ldg((const V *)((LOC ? gdiv_ : (const R *)a.divF) + (unsigned)(k0 + c) * strideK + own)), sx);
+    else if (EXT && a.divF) sx = P::add(sx, __ldg((const V *)((LOC ? gdiv_ : (const R *)a.divF) + (unsigned)(k0 + c) * strideK + own)));
     // FP64: the affine form (fewer FP64-pipe operations); FP32: U* first and
     // I* after the release (the FP32 kernels' register allocation prefers it)
     constexpr bool AFF = sizeof(R) == 8;
@@ -1511,12 +1513,12 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
     if (t < nc) {
       const int c = t, k = k0 + c;
       const unsigned cell = (unsigned)k * ncol + col;
-      if (ST2 && gsrc) {                  // stage 1's share of the source, added to in phase D
+      if (ST2 && a.src) {                  // stage 1's share of the source, added to in phase D
 #pragma unroll
-        for (int m = 0; m < 4; ++m) psrc[m] = gsrc[4 * cell + m];
+        for (int m = 0; m < 4; ++m) psrc[m] = source(cell)[m];
       }
       const double Tst = ST2 ? 0.5 * (a.T0[cell] + a.T1[cell]) : a.T0[cell];
-      const double aa = gaa[cell], as = gas_[cell];
+      const double aa = opac_a(cell), as = opac_s(cell);
       R rs[kNRedA] = {R(0), R(0), R(0)};
       for (int w = 0; w < nwarp; ++w)
 #pragma unroll
@@ -1534,7 +1536,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
         const double T2 = Tp * Tp;
         S = aa * a.a_rad * T2 * T2 + as * Ep;
       } else {
-        const double eta = geta[cell];
+        const double eta = emis(cell);
         const double den = 1.0 - A2 * as;
         ok = den > 0.0;
         const double Ep = (D + Em + kFourPi * A2 * eta) / den;
@@ -1550,15 +1552,15 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
     if (t < nc) {
       const unsigned cell = (unsigned)(k0 + t) * ncol + col;
       a.Tout[cell] = ST2 ? 0.5 * (a.T0[cell] + a.T1[cell]) : a.T0[cell];
-      if (gsrc && !ST2) {
-        for (int m = 0; m < 4; ++m) gsrc[4 * cell + m] = 0.0;
+      if (a.src && !ST2) {
+        for (int m = 0; m < 4; ++m) source(cell)[m] = 0.0;
       }
     }
   }
 
   // ---- phase C: implicit update of every bin
   V chk = zero;           // stays 0 unless a written value is not finite (0 * inf, 0 * nan = nan)
-  const bool want_src = couple && gsrc;
+  const bool want_src = couple && a.src;
   // I+ of one cell before the guard, from I* and the cell's source S
   auto implicit = [&](int c, V &Is, V &out) {
     Is = inpair ? *(const V *)(sI + c * nap + b0) : zero;
@@ -1709,7 +1711,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
         for (int w = 0; w < nwarp; ++w) s += red[(c * nwarp + w) * kNRedC + A];
         xs[A] = s;
       }
-      double *sp = gsrc + 4 * cell;
+      double *sp = source(cell);
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
         R dR = n0up * (cg.M[m][0] * xs[0] + cg.M[m][1] * xs[1] + cg.M[m][2] * xs[2] + cg.M[m][3] * xs[3]);
