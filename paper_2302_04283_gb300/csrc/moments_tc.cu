@@ -7,15 +7,33 @@
 // bf16(x), lo = bf16(x - hi), and D accumulates hi.hi + hi.lo + lo.hi in
 // FP32 (the lo.lo term is below 2^-16 relative).
 //
-// One CTA of 128 threads owns a tile of 128 cells (M = 128, one TMEM lane per
-// cell) and walks K in chunks of 64 bins: every thread converts its share of
-// the FP32 rows into bf16 hi/lo and stores them in the no-swizzle K-major
-// core-matrix layout (8 rows x 16 bytes per core matrix); one thread issues
-// 4 x 3 tcgen05.mma (M=128, N=16, K=16) into a TMEM accumulator and commits
-// to an mbarrier; after the last chunk each warp reads its 32 lanes back
-// with tcgen05.ld and writes the 10 components.  W^T hi/lo is built once on
-// the host and copied into shared memory per CTA.  Every wait is bounded: on
-// timeout the CTA records an error, frees its TMEM and returns.
+// One persistent CTA per SM walks tiles of 128 cells (M = 128, one TMEM lane
+// per cell) and K in chunks of 64 bins.  The kernel is bound by HBM (5 flop per
+// byte), so no part of the chain from load to output may wait for another:
+//   16 converter warps  hold their pieces of the next two chunks in registers
+//                       on their way (a warp's load covers two rows x 256
+//                       contiguous bytes), convert the arrived chunk into bf16
+//                       hi / lo and store it in the no-swizzle K-major
+//                       core-matrix layout (8 rows x 16 bytes per core matrix)
+//                       of one of two operand buffers;
+//   1 issuing warp      one thread issues up to 4 x 3 tcgen05.mma (M=128, N=16,
+//                       K=16) per chunk and commits to the buffer's mbarrier;
+//   4 epilogue warps    read a finished tile back (tcgen05.ld) from one of two
+//                       TMEM tiles, change the frame and write the components.
+// The K-direction stride of the core matrices is 2064 bytes (2048 + 16), which
+// spreads a warp's operand stores over all banks.  The previous form (four
+// CTAs of 128 threads, each loading, converting, issuing and waiting in turn)
+// left the memory idle meanwhile: 101 x 67 x 53 cells x 252 bins 0.145 -> 0.092 ms
+// (4.1 TB/s), with the same bits.  Tried on the way: all roles in 16 warps 0.146
+// ms (the issuing thread and the epilogue hold every chunk's barrier back),
+// 16-byte cp.async pieces 0.139 ms (every piece costs a 32-byte sector of L2),
+// 256-byte bulk copies 0.412 ms (some 80 cycles of an SM's copy engine each),
+// the weights' hi and lo side by side in one N = 32 MMA 0.088 ms (fluid-frame
+// components up to 1.3 times further from their 64-bit values: not kept).
+// W^T hi/lo is built once on the host; each chunk's 4 KB of it (from L2) travel
+// with the chunk, so shared memory does not grow with the bins.
+// Every wait is bounded: on timeout the CTA records an error, frees its TMEM
+// and returns.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -29,15 +47,22 @@ namespace rad {
 constexpr int kTcM = 128;           // cells per tile
 constexpr int kTcN = 16;            // moment columns (10 used)
 constexpr int kTcKC = 64;           // bins per K chunk
-constexpr int kTcThreads = 128;
+constexpr int kTcConv = 512;         // converter threads
+constexpr int kTcThreads = kTcConv + 32 + 128;
+constexpr int kTcDepth = 3;         // chunks a thread holds: two on their way, one being converted
+constexpr int kTcMaxKp = 2624;      // padded bins taken
+constexpr uint32_t kBChunk = kTcKC * kTcN * 2 * 2;     // hi then lo: one 16-byte piece per thread
+static_assert(kBChunk == kTcConv / 2 * 16, "one piece of W^T for half the threads");
+constexpr int kTcPieces = kTcM * kTcKC / 4 / kTcConv;   // 16-byte pieces per thread and chunk
 constexpr int kTcErrTimeout = 1 << 3;  // reported as RAD_ECUDA by rad_check
 constexpr long long kTcSpinLimit = 1ll << 24;
 
 // byte offsets of the K-major no-swizzle layouts
-//   A (128 x 64 chunk): core (mg, kg) at (kg * 16 + mg) * 128  -> SBO 128, LBO 2048
-//   B (16 x Kp):        core (ng, kg) at (kg * 2 + ng) * 128   -> SBO 128, LBO 256
-constexpr uint32_t kALbo = 2048, kASbo = 128, kBLbo = 256, kBSbo = 128;
-constexpr uint32_t kATile = kTcM * kTcKC * 2;   // 16 KB per operand half
+//   A (128 x 64 chunk): core (mg, kg) at kg * 2064 + mg * 128  -> SBO 128, LBO 2064
+//   B (16 x 64 chunk):  core (ng, kg) at (kg * 2 + ng) * 128   -> SBO 128, LBO 256
+constexpr uint32_t kALbo = 2064, kASbo = 128, kBLbo = 256, kBSbo = 128;
+constexpr uint32_t kATile = 8 * kALbo;          // one operand half (16 KB and the padding)
+static_assert(kATile % 128 == 0, "operand halves start on core matrix boundaries");
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -71,42 +96,50 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
         : "r"(bar), "r"(parity)
         : "memory");
     if (done) return true;
-    if ((it & 255) == 0) {                       // bounded in time as well as in polls
+    // bounded in time as well as in polls; the global timer takes about a
+    // microsecond to read, so only once a wait is long
+    if ((it & 63) == 63) {
       unsigned long long now;
       asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-      if (it == 0) t0 = now;
+      if (it == 63) t0 = now;
       else if (now - t0 > 2000000000ull) return false;
     }
   }
   return false;
 }
 
+// bf16 pair (low half a), rounded to nearest
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
   uint32_t r;
-  memcpy(&r, &v, 4);
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
   return r;
 }
 
-__global__ void __launch_bounds__(kTcThreads) k_moments_tc(const float *__restrict__ I, float *__restrict__ out,
-                                                         long long ncell, int nap, int nang, int kp,
-                                                         const uint4 *__restrict__ wt, int frame,
-                                                         const ColGeoF *cols, int ncol, const double *u,
-                                                         int *err) {
+__global__ void __launch_bounds__(kTcThreads, 1) k_moments_tc(const float *__restrict__ I, float *__restrict__ out,
+                                                            long long ncell, int nap, int nang, int kp,
+                                                            const uint4 *__restrict__ wt, int frame,
+                                                            const ColGeoF *cols, int ncol, const double *u,
+                                                            int *err) {
   extern __shared__ __align__(1024) unsigned char sm[];
-  unsigned char *Ah = sm;                    // [kATile]
-  unsigned char *Al = sm + kATile;           // [kATile]
-  unsigned char *Bw = sm + 2 * kATile;       // hi then lo, kp * 16 * 2 bytes each
-  const uint32_t bbytes = (uint32_t)kp * kTcN * 2;
-  uint64_t *bar = (uint64_t *)(Bw + 2 * bbytes);
-  uint32_t *tslot = (uint32_t *)(bar + 1);
-  const int t = threadIdx.x, warp = t >> 5;
-
-  // W^T hi / lo (prebuilt layout) into shared memory
-  const int nvec = (int)(2 * bbytes / 16);
-  for (int v = t; v < nvec; v += kTcThreads) ((uint4 *)Bw)[v] = wt[v];
+  // operand buffers [2][hi, lo][kATile], W^T chunks [2]
+  unsigned char *Aop = sm;
+  unsigned char *Bw = sm + 4 * kATile;
+  uint64_t *fullA = (uint64_t *)(Bw + 2 * kBChunk);      // per operand buffer: written (one arrival per converter warp)
+  uint64_t *emptyA = fullA + 2;                          // ... read by the tensor cores
+  uint64_t *fullD = emptyA + 2;                          // per TMEM tile: complete
+  uint64_t *emptyD = fullD + 2;                          // ... read back (one arrival per epilogue warp)
+  uint32_t *tslot = (uint32_t *)(emptyD + 2);
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   if (t == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)));
+    auto init = [](uint64_t *b, uint32_t n) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(b)), "r"(n));
+    };
+    for (int b = 0; b < 2; ++b) {
+      init(fullA + b, kTcConv / 32);
+      init(emptyA + b, 1);
+      init(fullD + b, 1);
+      init(emptyD + b, 4);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -117,111 +150,140 @@ __global__ void __launch_bounds__(kTcThreads) k_moments_tc(const float *__restri
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
-  const uint32_t sAh = smem_addr(Ah), sAl = smem_addr(Al), sBh = smem_addr(Bw), sBl = smem_addr(Bw + bbytes);
-  uint32_t phase = 0;
-  bool failed = false;
+  const uint32_t sA = smem_addr(Aop), sB = smem_addr(Bw);
+  auto arrive = [](uint64_t *b) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(b)) : "memory");
+  };
+  auto commit = [](uint64_t *b) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(b))
+                 : "memory");
+  };
 
   const long long ntile = (ncell + kTcM - 1) / kTcM;
-  constexpr int kSeg = (kTcM * kTcKC / 8) / kTcThreads;   // 8-bin segments per thread and chunk
-  // segment s of a chunk: cell m of the tile, bins kseg * 8 .. + 7 of the chunk
-  auto seg_m = [&](int it) { const int s = it * kTcThreads + t, g = s >> 5; return (g >> 1) * 8 + ((s & 31) >> 2); };
-  auto seg_k = [&](int it) { const int s = it * kTcThreads + t, g = s >> 5; return (g & 1) * 4 + (s & 3); };
-  // global loads of one chunk into registers (zeros outside the grid and the bins)
-  float4 v[2 * kSeg];
-  auto load = [&](long long tile, int k0) {
-#pragma unroll
-    for (int it = 0; it < kSeg; ++it) {
-      const long long cell = tile * kTcM + seg_m(it);
-      const int k = k0 + seg_k(it) * 8;
-      const float *row = I + cell * nap;
-      v[2 * it] = (cell < ncell && k < nap) ? __ldg((const float4 *)(row + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
-      v[2 * it + 1] = (cell < ncell && k + 4 < nap) ? __ldg((const float4 *)(row + k + 4))
-                                                    : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-  };
-  // split into bf16 hi / lo in the K-major core-matrix layout
-  auto convert = [&](int k0) {
-#pragma unroll
-    for (int it = 0; it < kSeg; ++it) {
-      const int m = seg_m(it), kseg = seg_k(it), k = k0 + kseg * 8;
-      float x[8] = {v[2 * it].x, v[2 * it].y, v[2 * it].z, v[2 * it].w,
-                    v[2 * it + 1].x, v[2 * it + 1].y, v[2 * it + 1].z, v[2 * it + 1].w};
-#pragma unroll
-      for (int e = 0; e < 8; ++e)
-        if (k + e >= nang) x[e] = 0.0f;                 // padding bins are not data
-      uint32_t h[4], l[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        __nv_bfloat16 h0 = __float2bfloat16_rn(x[2 * e]), h1 = __float2bfloat16_rn(x[2 * e + 1]);
-        float r0 = x[2 * e] - __bfloat162float(h0), r1 = x[2 * e + 1] - __bfloat162float(h1);
-        __nv_bfloat162 hh;
-        hh.x = h0;
-        hh.y = h1;
-        memcpy(&h[e], &hh, 4);
-        l[e] = pack_bf16(r0, r1);
-      }
-      const uint32_t off = (uint32_t)(kseg * 16 + (m >> 3)) * 128u + (uint32_t)(m & 7) * 16u;
-      *(uint4 *)(Ah + off) = make_uint4(h[0], h[1], h[2], h[3]);
-      *(uint4 *)(Al + off) = make_uint4(l[0], l[1], l[2], l[3]);
-    }
-  };
+  const int nk = kp / kTcKC;                                        // chunks per tile
+  const int mytiles = ntile > blockIdx.x ? (int)((ntile - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
+  const int nunit = mytiles * nk;                                   // this CTA's chunks
+  const long long row_step = (long long)gridDim.x * kTcM;
+  bool ok = true;
 
-  // software pipeline over (tile, chunk) units: the loads of the next unit are
-  // in flight while the tensor cores work on the current one
-  long long tile = blockIdx.x;
-  int k0 = 0;
-  if (tile < ntile) load(tile, k0);
-  while (tile < ntile && !failed) {
-    convert(k0);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    if (t == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (warp < kTcConv / 32) {
+    // ---- converters.  Piece `it` of a chunk: row it 32 + m0 of the tile, bins
+    // pk .. pk + 3 of the chunk (a warp: two rows x sixteen pieces)
+    const int m0 = warp * 2 + (lane >> 4), pk = (lane & 15) * 4;
+    const size_t prow = (size_t)32 * nap;
+    float4 v[kTcDepth][kTcPieces];
+    uint4 wv[kTcDepth];
+    long long left = ncell - (long long)blockIdx.x * kTcM - m0;     // rows from the first piece's on
+    const float *src = I + ((long long)blockIdx.x * kTcM + m0) * nap + pk;
+    const size_t tile_step = (size_t)row_step * nap - (size_t)nk * kTcKC;
+    const uint4 *wsrc = wt + (size_t)(t >> 7) * kp * kTcN * 2 / 16 + (t & 127);
+    int lkq = 0, lun = 0;
+    auto load = [&](float4 (&p)[kTcPieces], uint4 &w) {             // the next unit
+      if (lun >= nunit) return;
+      const bool kin = lkq * kTcKC + pk < nap;
 #pragma unroll
-      for (int kk = 0; kk < kTcKC / 16; ++kk) {
-        const uint32_t kb = (uint32_t)((k0 / 16 + kk) * 2) * kBLbo;   // 2 core matrices per K step
-        const uint64_t ah = umma_desc(sAh + kk * 2 * kALbo, kALbo, kASbo);
-        const uint64_t al = umma_desc(sAl + kk * 2 * kALbo, kALbo, kASbo);
-        const uint64_t bh = umma_desc(sBh + kb, kBLbo, kBSbo);
-        const uint64_t bl = umma_desc(sBl + kb, kBLbo, kBSbo);
-        const uint32_t first = (k0 == 0 && kk == 0) ? 0u : 1u;
-        mma_bf16(tmem, ah, bh, first);
-        mma_bf16(tmem, ah, bl, 1u);
-        mma_bf16(tmem, al, bh, 1u);
+      for (int it = 0; it < kTcPieces; ++it)
+        p[it] = kin && it * 32 < left ? __ldg((const float4 *)(src + it * prow)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      // this chunk's W^T: hi (threads 0 .. 127) and lo (128 .. 255)
+      if (t < kTcConv / 2) w = __ldg(wsrc + lkq * (kBChunk / 32));
+      ++lun;
+      src += kTcKC;
+      if (++lkq == nk) {
+        lkq = 0;
+        src += tile_step;
+        left -= row_step;
       }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       smem_addr(bar))
-                   : "memory");
+    };
+    const uint32_t off0 = (uint32_t)(pk >> 3) * kALbo + (uint32_t)(m0 >> 3) * 128u + (uint32_t)(m0 & 7) * 16u + (pk & 4) * 2u;
+    int kq = 0;
+    auto convert = [&](const float4 (&p)[kTcPieces], const uint4 &w, int buf) {
+      unsigned char *Ah = Aop + buf * 2 * kATile + off0;
+      const int k = kq * kTcKC + pk;
+#pragma unroll
+      for (int it = 0; it < kTcPieces; ++it) {
+        float4 x = p[it];
+        if (k + 3 >= nang) {                                // padding bins are not data
+          if (k >= nang) x.x = 0.0f;
+          if (k + 1 >= nang) x.y = 0.0f;
+          if (k + 2 >= nang) x.z = 0.0f;
+          x.w = 0.0f;
+        }
+        const uint32_t h0 = pack_bf16(x.x, x.y), h1 = pack_bf16(x.z, x.w);
+        const uint32_t l0 = pack_bf16(x.x - __uint_as_float(h0 << 16), x.y - __uint_as_float(h0 & 0xffff0000u));
+        const uint32_t l1 = pack_bf16(x.z - __uint_as_float(h1 << 16), x.w - __uint_as_float(h1 & 0xffff0000u));
+        *(uint2 *)(Ah + it * 512) = make_uint2(h0, h1);            // 32 rows on: four core matrices
+        *(uint2 *)(Ah + kATile + it * 512) = make_uint2(l0, l1);
+      }
+      if (t < kTcConv / 2) *(uint4 *)(Bw + buf * kBChunk + t * 16) = w;
+    };
+#pragma unroll
+    for (int s = 0; s < kTcDepth - 1; ++s) load(v[s], wv[s]);
+    for (int u0 = 0; u0 < nunit && ok; u0 += kTcDepth) {
+#pragma unroll
+      for (int s = 0; s < kTcDepth; ++s) {                        // static register slots
+        const int un = u0 + s, buf = un & 1;
+        if (un >= nunit || !ok) break;
+        load(v[(s + kTcDepth - 1) % kTcDepth], wv[(s + kTcDepth - 1) % kTcDepth]);
+        // the MMAs that read this operand buffer two units ago are done
+        ok = un < 2 || mbar_wait(smem_addr(emptyA + buf), (uint32_t)((un >> 1) - 1) & 1u);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        convert(v[s], wv[s], buf);
+        if (++kq == nk) kq = 0;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) arrive(fullA + buf);
+      }
     }
-    // next unit's loads, then wait for the MMAs (they read shared memory)
-    const long long cur_tile = tile;
-    const int cur_k0 = k0;
-    k0 += kTcKC;
-    if (k0 >= kp) {
-      k0 = 0;
-      tile += gridDim.x;
+  } else if (warp == kTcConv / 32) {
+    // ---- issuing thread
+    if (lane == 0) {
+      int un = 0;
+      for (int ti = 0; ti < mytiles && ok; ++ti) {
+        const uint32_t tcol = tmem + (uint32_t)(ti & 1) * kTcN;
+        // the tile read back from these columns two tiles ago
+        ok = ti < 2 || mbar_wait(smem_addr(emptyD + (ti & 1)), (uint32_t)((ti >> 1) - 1) & 1u);
+        for (int kq = 0; kq < nk && ok; ++kq, ++un) {
+          const int buf = un & 1;
+          ok = mbar_wait(smem_addr(fullA + buf), (uint32_t)(un >> 1) & 1u);
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const int steps = min(kTcKC / 16, (nang - kq * kTcKC + 15) / 16);    // K steps that hold data
+          uint64_t ah = umma_desc(sA + (uint32_t)buf * 2u * kATile, kALbo, kASbo);
+          uint64_t bh = umma_desc(sB + (uint32_t)buf * kBChunk, kBLbo, kBSbo);
+          constexpr uint64_t dl = kATile >> 4, da = (2 * kALbo) >> 4, dbl = (kBChunk / 2) >> 4, db = (2 * kBLbo) >> 4;
+          for (int kk = 0; kk < steps; ++kk, ah += da, bh += db) {   // 2 core matrices per K step
+            mma_bf16(tcol, ah, bh, (kq == 0 && kk == 0) ? 0u : 1u);
+            mma_bf16(tcol, ah, bh + dbl, 1u);
+            mma_bf16(tcol, ah + dl, bh, 1u);
+          }
+          commit(emptyA + buf);
+          if (kq == nk - 1) commit(fullD + (ti & 1));
+        }
+      }
+      // let the MMAs in flight end (again with a limit)
+      if (!ok && un > 0) mbar_wait(smem_addr(emptyA + ((un - 1) & 1)), (uint32_t)((un - 1) >> 1) & 1u);
     }
-    if (tile < ntile) load(tile, k0);
-    const bool ok = mbar_wait(smem_addr(bar), phase);
-    phase ^= 1u;
-    if (__syncthreads_or(!ok)) {   // the decision is uniform across the CTA
-      if (t == 0) atomicOr(err, kTcErrTimeout);
-      failed = true;
-      break;
-    }
-    if (cur_k0 + kTcKC < kp) continue;     // the tile has more chunks
-    const long long cell0 = cur_tile * kTcM;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // ---- epilogue: lane m of TMEM holds the 16 sums of cell cell0 + m
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(tmem + ((uint32_t)(warp * 32) << 16)));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    const long long cell = cell0 + t;
-    if (cell < ncell) {
+  } else {
+    // ---- epilogue: lane m of a tile's TMEM columns holds the 16 sums of its cell m
+    const int ew = warp & 3;                               // TMEM lanes 32 ew .. + 31 are this warp's
+    for (int ti = 0; ti < mytiles; ++ti) {
+      ok = mbar_wait(smem_addr(fullD + (ti & 1)), (uint32_t)(ti >> 1) & 1u);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      uint32_t r[16];
+      __syncwarp();
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+            "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+          : "r"(tmem + (uint32_t)(ti & 1) * kTcN + ((uint32_t)(ew * 32) << 16)));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      if (lane == 0) arrive(emptyD + (ti & 1));
+      const long long cell = (blockIdx.x + (long long)ti * gridDim.x) * kTcM + ew * 32 + lane;
+      if (cell >= ncell) continue;
       float Rt[10];
 #pragma unroll
       for (int p = 0; p < 10; ++p) Rt[p] = __uint_as_float(r[p]);
@@ -270,10 +332,9 @@ __global__ void __launch_bounds__(kTcThreads) k_moments_tc(const float *__restri
 #pragma unroll
       for (int p = 0; p < 10; ++p) o[p] = Ro[p];
     }
-    // all lanes have read TMEM before the next tile's first MMA overwrites it
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
   }
+  if (!ok) atomicOr(err, kTcErrTimeout);
+  __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;" ::"r"(tmem));
@@ -337,13 +398,12 @@ int launch_moments_bf16x3(rad_ctx *ctx, const float *I, int frame, const double 
     if (st != RAD_OK) return st;
   }
   const long long ncell = (long long)G.n[0] * G.n[1] * G.n[2];
-  // operands (hi, lo) + W^T (hi, lo) + barrier and TMEM slot
-  size_t smem = 2 * (size_t)kATile + 2 * (size_t)kp * kTcN * 2 + 64;
-  smem = (smem + 1023) / 1024 * 1024;
-  if (smem > 200 * 1024) {
-    err = "split-bf16 moments: too many bins for shared memory";
+  if (kp > kTcMaxKp) {
+    err = "split-bf16 moments: too many bins";
     return RAD_EUNSUPPORTED;
   }
+  // two operand buffers (hi, lo), two W^T chunks, barriers and TMEM slot
+  constexpr size_t smem = 4 * (size_t)kATile + 2 * kBChunk + 128;
   cudaError_t ce = cudaFuncSetAttribute(k_moments_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (ce != cudaSuccess) {
     err = std::string("split-bf16 moments: ") + cudaGetErrorString(ce);
@@ -353,8 +413,7 @@ int launch_moments_bf16x3(rad_ctx *ctx, const float *I, int frame, const double 
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   long long ntile = (ncell + kTcM - 1) / kTcM;
-  // four resident CTAs per SM keep enough loads in flight for HBM
-  long long blocks = std::min<long long>(ntile, (long long)nsm * 4);
+  const long long blocks = std::min<long long>(ntile, nsm);        // one persistent CTA per SM
   k_moments_tc<<<(unsigned)blocks, kTcThreads, smem, st>>>(I, R, ncell, ctx->ang.n_ap, ctx->ang.n_ang, kp,
                                                                      (const uint4 *)ctx->wt_dev, frame, G.colsF,
                                                                      G.n[0] * G.n[1], u, ctx->err_word);
