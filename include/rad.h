@@ -212,7 +212,10 @@ int rad_cfl_dt(rad_ctx *ctx, double cfl, double *dt_out);
  * coupling.  I (device, layout above) and gas->T are updated in place.
  * gas_src (device [k][j][i][4], nullable) receives -(dR^1/2 + dR^2), the
  * RK-weighted change of R^0_mu from the two couplings (the gas's share).
- * Allocates its stage scratch (one intensity array) on first use.
+ * Allocates its stage scratch (one intensity array) on first use, and on a
+ * spherical metric a table of the angular-flux prefactors per precision (7
+ * values per column and bin, FP64 also 2 per face; not beyond 4 GiB, and not
+ * while the stream is captured: the same results without it).
  * Geodesic levels up to 9 (812 bins: one CTA of at most 512 threads holds
  * every bin of a cell) and fewer than 2^32 intensity elements per block;
  * RAD_EUNSUPPORTED otherwise.

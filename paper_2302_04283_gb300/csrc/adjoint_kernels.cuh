@@ -234,14 +234,21 @@ __device__ __forceinline__ void slope_grad_of(float dl, float dr, float d[3]) {
 __device__ __forceinline__ void slope_grad_of(double dl, double dr, double d[3]) {
   const double r = rcp_digits(dl + dr), a = dr * r, b = dl * r;
   d[0] = -a * a;
-  d[1] = a - b;
+  d[1] = (dr - dl) * r;
   d[2] = b * b;
+}
+__device__ __forceinline__ bool one_sign(float dl, float dr) { return dl * dr > 0.0f; }
+// on the integer pipe; a zero (or subnormal) difference has no slope, as in the
+// forward kernel
+__device__ __forceinline__ bool one_sign(double dl, double dr) {
+  return (__double2hiint(dl) ^ __double2hiint(dr)) >= 0 && (__double2hiint(dl) & 0x7ff00000) != 0 &&
+         (__double2hiint(dr) & 0x7ff00000) != 0;
 }
 template <typename R>
 __device__ __forceinline__ void slope_grad(R v0, R v1, R v2, R d[3]) {
   const R dl = v1 - v0, dr = v2 - v1;
   d[0] = d[1] = d[2] = R(0);
-  if (dl * dr > R(0)) slope_grad_of(dl, dr, d);
+  if (one_sign(dl, dr)) slope_grad_of(dl, dr, d);
 }
 
 // Transposed transport of the inner cells (adj_inner_*) for DC and PLM
@@ -305,9 +312,14 @@ __global__ void __launch_bounds__(sizeof(R) == 8 ? 512 : 832) k_transport_adj_in
       if (d >= a.ndim || !act) continue;
       int f = yd + t - 1;                       // face between positions t - 2 and t - 1
       f = f < 0 ? f + N : (f >= N && a.bc_lo[d] == RAD_BC_PERIODIC ? f - N : f);
-      const Face &F = d == 0 ? ((const Face *)a.f1)[j * (a.n1 + 1) + f] : ((const Face *)a.f2)[f * a.n1 + i];
+      const int fi = d == 0 ? j * (a.n1 + 1) + f : f * a.n1 + i;
       bool u;
-      cA[d][t] = face_coefA(F, x, y, z, u);
+      if (sizeof(R) == 8 && a.face_c[d]) {
+        cA[d][t] = (R)a.face_c[d][(size_t)fi * a.nap + n] * ((const Face *)(d == 0 ? a.f1 : a.f2))[fi].dA;
+        u = a.face_up[d][(size_t)fi * a.nap + n];
+      } else {
+        cA[d][t] = face_coefA(((const Face *)(d == 0 ? a.f1 : a.f2))[fi], x, y, z, u);
+      }
       up[d] |= (u ? 1u : 0u) << t;
     }
   }
@@ -336,8 +348,15 @@ __global__ void __launch_bounds__(sizeof(R) == 8 ? 512 : 832) k_transport_adj_in
       slope_grad<R>(v[2], v[3], v[4], dp);
     }
     R lp[4];
+    if (sizeof(R) == 8) {           // the cells' mu / dV once each
+      R m[5];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
+      for (int t = 0; t < 5; ++t) m[t] = ivd[t] * mm[t];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) lp[t] = cA[d][t] * (m[t + 1] - m[t]);
+    }
+#pragma unroll
+    for (int t = 0; t < 4 && sizeof(R) == 4; ++t) {
       lp[t] = fma_rn(mul_rn(cA[d][t], ivd[t + 1]), mm[t + 1], mul_rn(mul_rn(-cA[d][t], ivd[t]), mm[t]));
     }
     // face 0 holds the cell only in the slope of its right cell, face 3 only

@@ -343,6 +343,10 @@ void free_geometry(DevGeom &g) {
     cudaFree(g.side_up[p]);
     g.side_P[p] = nullptr;
     g.side_up[p] = nullptr;
+    cudaFree(g.face_c[p]);
+    cudaFree(g.face_up[p]);
+    g.face_c[p] = nullptr;
+    g.face_up[p] = nullptr;
   }
   g.cols = nullptr;
   g.f1 = g.f2 = g.f3 = nullptr;

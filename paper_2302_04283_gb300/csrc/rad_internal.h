@@ -128,6 +128,11 @@ struct DevGeom {
   // set where the bin is upwind of its side s
   void *side_P[2] = {nullptr, nullptr};
   unsigned char *side_up[2] = {nullptr, nullptr};
+  // FP64 only, built with it: n^d n_0 of every x1 face [n2][n1+1][n_ap]
+  // (index 0) and x2 face [n2+1][n1][n_ap] (1), and whether n^d < 0 (the
+  // upwind cell is the upper one)
+  double *face_c[2] = {nullptr, nullptr};
+  unsigned char *face_up[2] = {nullptr, nullptr};
 };
 
 }  // namespace rad

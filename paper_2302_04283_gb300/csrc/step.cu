@@ -177,6 +177,11 @@ StageArgs make_stage_args(rad_ctx *ctx, const rad_gas *gas, double dt, const rad
   a.nbr_t = ctx->dang.nbr_t;
   a.rslot_t = ctx->dang.rslot_t;
   a.rdO = ctx->dang.rdO;
+  for (int d = 0; d < 2; ++d) {
+    const bool both = G.face_c[0] && G.face_c[1];
+    a.face_c[d] = both ? G.face_c[d] : nullptr;
+    a.face_up[d] = both ? G.face_up[d] : nullptr;
+  }
   a.side_P = G.side_P[o->precision == RAD_F32];
   a.side_up = G.side_up[o->precision == RAD_F32];
   a.edge_pq = ctx->dang.edge_pq;

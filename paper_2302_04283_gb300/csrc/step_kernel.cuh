@@ -79,6 +79,8 @@ struct StageArgs {
   const double *rdO;       // 1 / dOmega
   const void *side_P;      // side table of this precision (null: formed by the kernels)
   const unsigned char *side_up;
+  const double *face_c[2];         // FP64: tabulated n^d n_0 of the x1 and x2 faces (null: formed by the kernels)
+  const unsigned char *face_up[2];
   const int *edge_line;    // latitude-longitude grids: cell behind p, cell beyond q of each side
   const int *line_behind;  // latitude-longitude grids: per bin, the sides it is the cell behind of (adjoint)
   int n_edge;              // sides of the angle grid
@@ -842,6 +844,14 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
       upR = (nd.x < R(0) ? 1u : 0u) | (nd.y < R(0) ? 2u : 0u);
       const R f = F.m0[0] * F.dA * invdV;
       return P::mk(act0 ? nd.x * f : R(0), act1 ? nd.y * f : R(0));
+    }
+    if (sizeof(R) == 8 && d < 2 && a.face_c[d]) {
+      const size_t fi = (size_t)(&F - (const Face *)(d == 0 ? a.f1 : a.f2)) * nap + (inpair ? b0 : 0);
+      const double2 c = __ldg((const double2 *)(a.face_c[d] + fi));
+      const uchar2 u = *(const uchar2 *)(a.face_up[d] + fi);
+      upR = (u.x ? 1u : 0u) | (u.y ? 2u : 0u);
+      const R f = F.dA * invdV;
+      return P::mk(act0 ? (R)c.x * f : R(0), act1 ? (R)c.y * f : R(0));
     }
     V na = P::fma(nhz, P::mk(F.ea[3], F.ea[3]),
                   P::fma(nhy, P::mk(F.ea[2], F.ea[2]), P::fma(nhx, P::mk(F.ea[1], F.ea[1]), P::mk(F.ea[0], F.ea[0]))));
