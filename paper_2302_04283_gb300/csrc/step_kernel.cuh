@@ -704,7 +704,6 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
   const int nap = NAP > 0 ? NAP : (NAP < 0 ? -NAP : a.nap);   // padded bins per row
   const int t = threadIdx.x;
   const int ncons = blockDim.x - 32;                      // consumer threads; the last warp produces
-  const bool cons = t < ncons;
   const int nwarp = ncons >> 5;                           // consumer warps
   const int lane = t & 31, warp = t >> 5;
   const int b0 = 2 * t;                                   // bins b0, b0 + 1
@@ -755,7 +754,129 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
   uint64_t *bars = (uint64_t *)(((uintptr_t)(gbuf + (AM ? 4 * nap : 0)) + 15) & ~(uintptr_t)15);   // [depth] full
   uint64_t *ebars = bars + kMaxStages;                                                // [depth] empty
 
-  for (int c = t; c < nc; c += blockDim.x) {
+  // ---- stencil rows of one cell (h = 2, or 3 for PPM): the contiguous x1
+  // block (rows i-h..i+h, or one copy per row at a boundary), the 2h x2 rows,
+  // this column's row at k+h (x3 window) and, in stage 2, this column's row
+  // of I^0.  Slots: 0..2h x1 block (h = own), then the x2 rows j-h..j+h
+  // without j, then own k+h, then I^0.
+  // row kinds (wrap_idx): x1 rows 0 or a halo side (2, 3); x2 rows 0, the
+  // polar mirror (1) or a halo side
+  int xs[X1N], xk[X1N], yj[X2N], ypol[X2N];
+  bool x1contig = true;
+  for (int q = 0; q < X1N; ++q) {
+    int kind = 0;
+    xs[q] = q == H ? i : wrap_idx<EXT>(i + q - H, a.n1, a.bc_lo[0], a.bc_hi[0], kind);
+    xk[q] = kind;
+    if (xs[q] != i + q - H || (EXT && kind)) x1contig = false;
+  }
+  bool anypol = false;
+  for (int q = 0; q < X2N; ++q) {
+    int pol = 0;
+    const int o = q < H ? q - H : q - H + 1;
+    yj[q] = a.ndim >= 2 ? wrap_idx<EXT>(j + o, a.n2, a.bc_lo[1], a.bc_hi[1], pol) : j;
+    ypol[q] = pol;
+    anypol |= pol == 1;
+  }
+  const bool d3 = a.ndim >= 3;
+  const size_t rowb = (size_t)nap * sizeof(R);
+  auto rowp = [&](const R *base, int ii, int jj, int kk) {
+    return base + ((size_t)kk * ncol + (size_t)jj * a.n1 + ii) * nap;
+  };
+  // this column's row at plane k (any k: wrapped, clamped or a halo row)
+  auto kidx = [&](int k) {
+    int kind;
+    return wrap_idx<EXT>(k, a.n3, a.bc_lo[2], a.bc_hi[2], kind);
+  };
+  auto krow = [&](int k) -> const R * {
+    int kind;
+    const int kk = wrap_idx<EXT>(k, a.n3, a.bc_lo[2], a.bc_hi[2], kind);
+    if (EXT && kind >= 2) return halo_row<R>(a.halo, a.n1, a.n2, a.n3, 2, kind - 2, kk, i, j, 0, nap);
+    return rowp(Ip, i, j, kk);
+  };
+  auto produce = [&](int c, int st) {   // issue the copies of cell k0 + c into ring stage st
+    const int k = k0 + c;
+    R *dst = stg + (size_t)st * ROWS * nap;
+    uint32_t bytes = (uint32_t)(X1N * rowb) + (a.ndim >= 2 ? (uint32_t)(X2N * rowb) : 0u) +
+                     (d3 ? (uint32_t)rowb : 0u) + (ST2 ? (uint32_t)rowb : 0u);
+    mbar_expect_tx(&bars[st], bytes);
+    if (x1contig) {
+      bulk_g2s(dst, rowp(Ip, i - H, j, k), (uint32_t)(X1N * rowb), &bars[st]);
+    } else {
+      for (int q = 0; q < X1N; ++q) {
+        const R *src = (EXT && xk[q] >= 2) ? halo_row<R>(a.halo, a.n1, a.n2, a.n3, 0, xk[q] - 2, xs[q], 0, j, k, nap)
+                                           : rowp(Ip, xs[q], j, k);
+        bulk_g2s(dst + q * nap, src, (uint32_t)rowb, &bars[st]);
+      }
+    }
+    if (a.ndim >= 2) {
+      for (int q = 0; q < X2N; ++q) {
+        const R *src;
+        if (EXT && ypol[q] >= 2) {
+          src = halo_row<R>(a.halo, a.n1, a.n2, a.n3, 1, ypol[q] - 2, yj[q], i, 0, k, nap);
+        } else {
+          int kk = k;
+          if (ypol[q] == 1 && a.n3 > 1) kk = (k + a.n3 / 2) % a.n3;
+          src = rowp(Ip, i, yj[q], kk);
+        }
+        bulk_g2s(dst + (SX2 + q) * nap, src, (uint32_t)rowb, &bars[st]);
+      }
+    }
+    if (d3) bulk_g2s(dst + SX3 * nap, EXT ? krow(k + H) : rowp(Ip, i, j, kidx(k + H)), (uint32_t)rowb, &bars[st]);
+    if (ST2) bulk_g2s(dst + SI0 * nap, rowp(I0, i, j, k), (uint32_t)rowb, &bars[st]);
+  };
+  // ---- producer warp: one lane issues every cell's copies into the ring,
+  // waiting for the consumers to release a stage before refilling it.  In the
+  // run-time-row and block kernels (EARLY) it starts before the set-up, in which it takes
+  // no part, so that the first rows travel meanwhile (2D hot spot FP64 53.2 ->
+  // 43.4 us, lat/long 90 x 50 x 44 x 128 FP32 1.57 -> 1.47 ms, 61 x 37 x 34 x 92 FP64
+  // 3.66 -> 3.57); the fixed-row FP32 kernels lose by it (their registers are
+  // allocated otherwise: 128^3 x 162 6.81 -> 7.29 ms, 128 x 64 x 64 x 362 5.15 -> 5.24).
+  constexpr bool EARLY = EXT;
+  bool timeout = false;
+  auto init_bars = [&]() {
+    if (t == 0) {
+      for (int st = 0; st < a.depth; ++st) {
+        mbar_init(&bars[st], 1);
+        mbar_init(&ebars[st], (uint32_t)nwarp);
+      }
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();   // barriers initialised (and, where they come later, the gas staged)
+  };
+  auto run_producer = [&]() {
+    if (lane == 0) {
+      int st = 0;
+      uint32_t ph = 0;                      // parity of the empty barrier's next phase
+      for (int c = 0; c < nc; ++c) {
+        if (c >= a.depth && !mbar_wait_parity(&ebars[st], ph)) {
+          timeout = true;     // the consumers time out on the full barrier in turn
+          break;
+        }
+        produce(c, st);
+        if (++st == a.depth) {
+          st = 0;
+          if (c >= a.depth) ph ^= 1u;
+        }
+      }
+    }
+  };
+  if (EARLY) {
+    init_bars();
+    if (t >= ncons) {
+      run_producer();
+      if (timeout) atomicOr(a.err, 1 << 3);
+      __syncwarp();
+      // the CTA barriers of phases B to D
+      __syncthreads();
+      if (couple) __syncthreads();
+      if (couple && a.src) __syncthreads();
+      return;
+    }
+  }
+  const bool cons = EARLY || t < ncons;
+  const int nstage = EARLY ? ncons : blockDim.x;           // threads that stage the gas
+
+  for (int c = t; c < nc; c += nstage) {
     const unsigned cell = (unsigned)(k0 + c) * ncol + col;
     if (couple || tau) {
       const R ux = (R)a.u[3 * cell], uy = (R)a.u[3 * cell + 1], uz = (R)a.u[3 * cell + 2];
@@ -771,7 +892,7 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
     // optical-depth weighting (Sec. 2.4): per cell and face, the face's
     // f = -expm1(-tau^2) with tau = C alpha_E dt / u^0hat from the face
     // averages of u and alpha_E, and the neighbour's velocity (for its n^0bar)
-    for (int q = t; q < nc * 6; q += blockDim.x) {
+    for (int q = t; q < nc * 6; q += nstage) {
       const int c = q / 6, s = q % 6, d = s >> 1, sg = (s & 1) ? 1 : -1;
       R *o = stau + (c * 6 + s) * 5;
       if (d >= a.ndim) {
@@ -1092,76 +1213,6 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
         if (b0 + e < a.nang) a_self[e] = tab ? (e ? sv.y : sv.x) : per_solid_angle(a_self[e], a.dOmega, a.rdO, b0 + e);
     }
   }
-  // ---- stencil rows of one cell (h = 2, or 3 for PPM): the contiguous x1
-  // block (rows i-h..i+h, or one copy per row at a boundary), the 2h x2 rows,
-  // this column's row at k+h (x3 window) and, in stage 2, this column's row
-  // of I^0.  Slots: 0..2h x1 block (h = own), then the x2 rows j-h..j+h
-  // without j, then own k+h, then I^0.
-  // row kinds (wrap_idx): x1 rows 0 or a halo side (2, 3); x2 rows 0, the
-  // polar mirror (1) or a halo side
-  int xs[X1N], xk[X1N], yj[X2N], ypol[X2N];
-  bool x1contig = true;
-  for (int q = 0; q < X1N; ++q) {
-    int kind = 0;
-    xs[q] = q == H ? i : wrap_idx<EXT>(i + q - H, a.n1, a.bc_lo[0], a.bc_hi[0], kind);
-    xk[q] = kind;
-    if (xs[q] != i + q - H || (EXT && kind)) x1contig = false;
-  }
-  bool anypol = false;
-  for (int q = 0; q < X2N; ++q) {
-    int pol = 0;
-    const int o = q < H ? q - H : q - H + 1;
-    yj[q] = a.ndim >= 2 ? wrap_idx<EXT>(j + o, a.n2, a.bc_lo[1], a.bc_hi[1], pol) : j;
-    ypol[q] = pol;
-    anypol |= pol == 1;
-  }
-  const bool d3 = a.ndim >= 3;
-  const size_t rowb = (size_t)nap * sizeof(R);
-  auto rowp = [&](const R *base, int ii, int jj, int kk) {
-    return base + ((size_t)kk * ncol + (size_t)jj * a.n1 + ii) * nap;
-  };
-  // this column's row at plane k (any k: wrapped, clamped or a halo row)
-  auto kidx = [&](int k) {
-    int kind;
-    return wrap_idx<EXT>(k, a.n3, a.bc_lo[2], a.bc_hi[2], kind);
-  };
-  auto krow = [&](int k) -> const R * {
-    int kind;
-    const int kk = wrap_idx<EXT>(k, a.n3, a.bc_lo[2], a.bc_hi[2], kind);
-    if (EXT && kind >= 2) return halo_row<R>(a.halo, a.n1, a.n2, a.n3, 2, kind - 2, kk, i, j, 0, nap);
-    return rowp(Ip, i, j, kk);
-  };
-  auto produce = [&](int c, int st) {   // issue the copies of cell k0 + c into ring stage st
-    const int k = k0 + c;
-    R *dst = stg + (size_t)st * ROWS * nap;
-    uint32_t bytes = (uint32_t)(X1N * rowb) + (a.ndim >= 2 ? (uint32_t)(X2N * rowb) : 0u) +
-                     (d3 ? (uint32_t)rowb : 0u) + (ST2 ? (uint32_t)rowb : 0u);
-    mbar_expect_tx(&bars[st], bytes);
-    if (x1contig) {
-      bulk_g2s(dst, rowp(Ip, i - H, j, k), (uint32_t)(X1N * rowb), &bars[st]);
-    } else {
-      for (int q = 0; q < X1N; ++q) {
-        const R *src = (EXT && xk[q] >= 2) ? halo_row<R>(a.halo, a.n1, a.n2, a.n3, 0, xk[q] - 2, xs[q], 0, j, k, nap)
-                                           : rowp(Ip, xs[q], j, k);
-        bulk_g2s(dst + q * nap, src, (uint32_t)rowb, &bars[st]);
-      }
-    }
-    if (a.ndim >= 2) {
-      for (int q = 0; q < X2N; ++q) {
-        const R *src;
-        if (EXT && ypol[q] >= 2) {
-          src = halo_row<R>(a.halo, a.n1, a.n2, a.n3, 1, ypol[q] - 2, yj[q], i, 0, k, nap);
-        } else {
-          int kk = k;
-          if (ypol[q] == 1 && a.n3 > 1) kk = (k + a.n3 / 2) % a.n3;
-          src = rowp(Ip, i, yj[q], kk);
-        }
-        bulk_g2s(dst + (SX2 + q) * nap, src, (uint32_t)rowb, &bars[st]);
-      }
-    }
-    if (d3) bulk_g2s(dst + SX3 * nap, EXT ? krow(k + H) : rowp(Ip, i, j, kidx(k + H)), (uint32_t)rowb, &bars[st]);
-    if (ST2) bulk_g2s(dst + SI0 * nap, rowp(I0, i, j, k), (uint32_t)rowb, &bars[st]);
-  };
   const int p0 = act0 ? a.perm[b0] : 0, p1 = act1 ? a.perm[b0 + 1] : 0;
   const unsigned own = (unsigned)col * nap + (inpair ? b0 : 0);
   const int bb = inpair ? b0 : 0;
@@ -1169,33 +1220,11 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
   const R dtR = (R)a.dt, dts = (R)a.dts;
   const R c2pre = dts / R(kFourPi);
   const V zero = P::mk(R(0), R(0));
-  if (t == 0) {
-    for (int st = 0; st < a.depth; ++st) {
-      mbar_init(&bars[st], 1);
-      mbar_init(&ebars[st], (uint32_t)nwarp);
-    }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();   // gas staged, barriers initialised
-  bool timeout = false;
-  if (!cons) {
-    // ---- producer warp: one lane issues every cell's copies into the ring,
-    // waiting for the consumers to release a stage before refilling it
-    if (lane == 0) {
-      int st = 0;
-      uint32_t ph = 0;                      // parity of the empty barrier's next phase
-      for (int c = 0; c < nc; ++c) {
-        if (c >= a.depth && !mbar_wait_parity(&ebars[st], ph)) {
-          timeout = true;     // the consumers time out on the full barrier in turn
-          break;
-        }
-        produce(c, st);
-        if (++st == a.depth) {
-          st = 0;
-          if (c >= a.depth) ph ^= 1u;
-        }
-      }
-    }
+  if (EARLY) {
+    asm volatile("bar.sync 1, %0;" ::"r"(ncons) : "memory");     // gas staged (consumer warps)
+  } else {
+    init_bars();
+    if (!cons) run_producer();
   }
 
   // ---- phase A (consumer warps): transport, stage combination, primitive I*, coupling sums
