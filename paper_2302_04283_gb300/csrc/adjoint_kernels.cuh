@@ -261,8 +261,9 @@ __device__ __forceinline__ void slope_grad(R v0, R v1, R v2, R d[3]) {
 // window value through the boundary map.  x3 values ride in a register
 // window.  Bound by the FP64 pipe in FP64 and by the loads' latency in FP32;
 // one thread per bin, because 92 bins fill three warps of threads (96 %) but
-// two of pairs (72 %).  256 x 128 cells x 162 bins FP64 4.0 -> 2.0 ms per stage
-// (11.2 before the side table), 45 x 38 x 33 x 162 FP32 1.40 -> 0.74 ms.
+// two of pairs (72 %).  Per stage, with the boundary cells'
+// launch and the side table's share: 256 x 128 cells x 162 bins FP64 11.2 -> 1.87
+// + 0.30 ms, 45 x 38 x 33 x 162 FP32 1.40 -> 0.23 + 0.18 ms.
 template <typename R, bool ANG>
 __global__ void __launch_bounds__(sizeof(R) == 8 ? 512 : 832) k_transport_adj_in(AdjArgs A) {
   using Col = typename GeoTypes<R>::Col;

@@ -8,9 +8,9 @@
 // of the FP64 kernels.  It depends on the metric and the angle grid only, so
 // it is laid out once per context and precision, in the order the consumer
 // threads read it (bin fastest), and read back as one coalesced row per slot.
-// Per rad_step: Kerr-Schild 128 x 64 x 64 x 362 bins FP32 6.72 -> 5.15 ms
-// (192 x 96 x 96 x 642: 43.5 -> 32.3), 61 x 37 x 34 x 92 FP64 7.09 -> 5.69 ms,
-// 256 x 128 x 162 FP64 15.4 -> 5.0 ms.  Building it takes about as long as
+// Step and moments: Kerr-Schild 128 x 64 x 64 x 362 bins FP32 7.01 -> 5.45 ms
+// (192 x 96 x 96 x 642: 45.5 -> 34.2), 61 x 37 x 34 x 92 FP64 7.09 -> 5.69 ms,
+// 256 x 128 x 162 FP64 gradient over two steps 117.8 -> 47.3.  Building it takes about as long as
 // one stage gains by it.
 #include <algorithm>
 
