@@ -172,7 +172,8 @@ __device__ __forceinline__ R face_val(bool upR, bool plm, R a, R b, R c, R d) {
 // decreases monotonically onto the root.  The FP32 path gets close in FP32
 // and finishes with FP64 steps (Newton with a slope accurate to 1e-7 still
 // gains seven digits per step), falling back to the FP64 iteration when the
-// FP64 residual is not small; the FP64 path iterates in FP64 throughout.
+// FP64 residual is not small; the FP64 path (full64) with a guess starts the
+// same way and falls back when its last step is not a rounding's size.
 // guess > 0 (the temperature before the coupling, usually close to the
 // root): one Newton step from it first.  f is convex, so from either side
 // the step lands at or above the root; inside the bracket it replaces the
@@ -221,7 +222,11 @@ __device__ __forceinline__ double quartic_root(double B4, double B1, double B0, 
     // FP32 slope, each gaining six digits or more: 25 FP64 operations in place
     // of several Newton steps with correctly rounded divisions (a cell's solve
     // occupies the FP64 pipe like a whole warp's; in a 2D grid it runs per
-    // cell).  Kept if the last step is a rounding's size.
+    // cell).  Kept if the last step is a rounding's size and means something:
+    // an FP32 slope above 2^126 (or infinite, once T^3 or B1 leaves the FP32
+    // range) has the reciprocal 0 and the step is 0 wherever T is; below that the
+    // slope is within roundings of the FP64 one, so that a small step is a small
+    // distance from the root.
     const float b4f = (float)B4, b1f = (float)B1, b0f = (float)B0;
     float tf = fminf(-b0f / b1f, sqrtf(sqrtf(-b0f / b4f))), ifp = 0.0f;
     {
@@ -245,7 +250,7 @@ __device__ __forceinline__ double quartic_root(double B4, double B1, double B0, 
       d = fma(fma(B4, T2 * T, B1), T, B0) * sl;
       T -= d;
     }
-    if (T > 0.0 && fabs(d) <= 1e-15 * T) return T;
+    if (ifp > 0.0f && T > 0.0 && fabs(d) <= 1e-15 * T) return T;
   }
   // FP64: Newton from the upper bound decreases monotonically onto the root
   double T = fmin(-B0 / B1, sqrt(sqrt(-B0 / B4)));
