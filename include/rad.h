@@ -214,8 +214,8 @@ int rad_cfl_dt(rad_ctx *ctx, double cfl, double *dt_out);
  * RK-weighted change of R^0_mu from the two couplings (the gas's share).
  * Allocates its stage scratch (one intensity array) on first use, and on a
  * spherical metric a table of the angular-flux prefactors per precision (7
- * values per column and bin, FP64 also 2 per face; not beyond 4 GiB, and not
- * while the stream is captured: the same results without it).
+ * values per column and bin, FP64 also 2 per face; 4 GiB per precision at
+ * most, and not while the stream is captured: the same results without it).
  * Geodesic levels up to 9 (812 bins: one CTA of at most 512 threads holds
  * every bin of a cell) and fewer than 2^32 intensity elements per block;
  * RAD_EUNSUPPORTED otherwise.

@@ -339,12 +339,10 @@ void free_geometry(DevGeom &g) {
   cudaFree(g.f3F);
   cudaFree(g.xf_dev);
   for (int p = 0; p < 2; ++p) {
-    cudaFree(g.side_P[p]);
-    cudaFree(g.side_up[p]);
+    cudaFree(g.side_buf[p]);
+    g.side_buf[p] = nullptr;
     g.side_P[p] = nullptr;
     g.side_up[p] = nullptr;
-    cudaFree(g.face_c[p]);
-    cudaFree(g.face_up[p]);
     g.face_c[p] = nullptr;
     g.face_up[p] = nullptr;
   }

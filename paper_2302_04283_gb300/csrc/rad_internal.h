@@ -126,6 +126,8 @@ struct DevGeom {
   // sides, oriented out of the bin (0 where there is no side), row 6 the sum
   // of those whose upwind cell is the bin itself; side_up [col][n_ap], bit s
   // set where the bin is upwind of its side s
+  // one allocation per precision holds them
+  void *side_buf[2] = {nullptr, nullptr};
   void *side_P[2] = {nullptr, nullptr};
   unsigned char *side_up[2] = {nullptr, nullptr};
   // FP64 only, built with it: n^d n_0 of every x1 face [n2][n1+1][n_ap]

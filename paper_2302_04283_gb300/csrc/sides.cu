@@ -72,9 +72,11 @@ __global__ void k_face_table(const FaceGeo *__restrict__ faces, int nang, int na
 
 }  // namespace
 
-// The table's bound: 4 GiB per precision (a 2D grid of 460,000 columns with
-// 162 bins in FP64).  Beyond it, or when the allocation fails, or while the
-// stream is being captured, the kernels form the prefactors as they go.
+// The tables' bound: 4 GiB per precision, side and face tables and their flags
+// together (in FP64 a 2D grid of 350,000 columns with 162 bins).  Face tables
+// that do not fit beside the side table are left out.  Beyond the bound, or
+// when the allocation fails, or while the stream is being captured, the
+// kernels form the prefactors as they go.
 constexpr size_t kSideTableMax = (size_t)4 << 30;
 
 void ensure_side_table(rad_ctx *ctx, int precision) {
@@ -82,20 +84,30 @@ void ensure_side_table(rad_ctx *ctx, int precision) {
   const int ip = precision == RAD_F32 ? 1 : 0;
   if (G.kind == RAD_MINK_CART || G.side_P[ip]) return;
   const size_t ncol = (size_t)G.n[0] * G.n[1], nap = (size_t)ctx->ang.n_ap;
-  const size_t bytes = ncol * nap * kSideRows * (ip ? 4 : 8);      // and 2 / 7 more for the FP64 faces
-  if (bytes > kSideTableMax) return;
+  const size_t nf[2] = {(size_t)G.n[1] * (G.n[0] + 1), (size_t)(G.n[1] + 1) * G.n[0]};
+  auto pad = [](size_t b) { return (b + 255) / 256 * 256; };
+  const size_t bP = pad(ncol * nap * kSideRows * (ip ? 4 : 8)), bU = pad(ncol * nap);
+  // the FP64 kernels also read the faces' prefactors (eight operations of their
+  // pipe per bin and face: in a 2D grid, where a CTA has one cell, as much as a
+  // third of the update; two gradient steps of 256 x
+  // 128 x 162: 27.8 -> 24.3 ms with the adjoint's slopes on fewer operations)
+  size_t bF = 0;
+  for (int d = 0; d < 2 && !ip; ++d) bF += pad(nf[d] * nap * sizeof(double)) + pad(nf[d] * nap);
+  if (bP + bU + bF > kSideTableMax) bF = 0;
+  if (bP + bU > kSideTableMax) return;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
     return;
   }
-  void *P = nullptr;
-  unsigned char *up = nullptr;
-  if (cudaMalloc(&P, bytes) != cudaSuccess || cudaMalloc(&up, ncol * nap) != cudaSuccess) {
+  unsigned char *buf = nullptr;
+  while (cudaMalloc(&buf, bP + bU + bF) != cudaSuccess) {
     cudaGetLastError();
-    cudaFree(P);
-    return;
+    if (!bF) return;
+    bF = 0;
   }
+  void *P = buf;
+  unsigned char *up = buf + bP, *next = up + bU;
   const int threads = std::min(256, (int)(nap + 31) / 32 * 32);
   if (ip)
     k_side_table<float, ColGeoF><<<(unsigned)ncol, threads, 0, ctx->stream>>>(
@@ -105,36 +117,25 @@ void ensure_side_table(rad_ctx *ctx, int precision) {
     k_side_table<double, ColGeo><<<(unsigned)ncol, threads, 0, ctx->stream>>>(
         G.cols, ctx->ang.n_ang, (int)nap, ctx->dang.slot_nbr, ctx->dang.slot_edge, ctx->dang.edge_pq,
         ctx->dang.edge_geo, ctx->dang.dOmega, ctx->dang.rdO, (double *)P, up);
+  double *c[2] = {nullptr, nullptr};
+  unsigned char *u[2] = {nullptr, nullptr};
+  for (int d = 0; d < 2 && bF; ++d) {
+    c[d] = (double *)next;
+    u[d] = next + pad(nf[d] * nap * sizeof(double));
+    next = u[d] + pad(nf[d] * nap);
+    k_face_table<<<(unsigned)nf[d], threads, 0, ctx->stream>>>(d == 0 ? G.f1 : G.f2, ctx->ang.n_ang, (int)nap,
+                                                             ctx->dang.dir, c[d], u[d]);
+  }
   if (cudaGetLastError() != cudaSuccess) {
-    cudaFree(P);
-    cudaFree(up);
+    cudaFree(buf);
     return;
   }
+  G.side_buf[ip] = buf;
   G.side_P[ip] = P;
   G.side_up[ip] = up;
-  if (ip) return;
-  // the FP64 kernels also read the faces' prefactors (eight operations of their
-  // pipe per bin and face: in a 2D grid, where a CTA has one cell, as much as a
-  // third of the update; two gradient steps of 256 x
-  // 128 x 162: 27.8 -> 24.3 ms with the adjoint's slopes on fewer operations)
-  for (int d = 0; d < 2; ++d) {
-    const size_t nf = d == 0 ? (size_t)G.n[1] * (G.n[0] + 1) : (size_t)(G.n[1] + 1) * G.n[0];
-    double *c = nullptr;
-    unsigned char *u = nullptr;
-    if (cudaMalloc(&c, nf * nap * sizeof(double)) != cudaSuccess || cudaMalloc(&u, nf * nap) != cudaSuccess) {
-      cudaGetLastError();
-      cudaFree(c);
-      return;
-    }
-    k_face_table<<<(unsigned)nf, threads, 0, ctx->stream>>>(d == 0 ? G.f1 : G.f2, ctx->ang.n_ang, (int)nap,
-                                                          ctx->dang.dir, c, u);
-    if (cudaGetLastError() != cudaSuccess) {
-      cudaFree(c);
-      cudaFree(u);
-      return;
-    }
-    G.face_c[d] = c;
-    G.face_up[d] = u;
+  for (int d = 0; d < 2 && !ip; ++d) {
+    G.face_c[d] = c[d];
+    G.face_up[d] = u[d];
   }
 }
 
