@@ -341,6 +341,7 @@ void free_geometry(DevGeom &g) {
   for (int p = 0; p < 2; ++p) {
     cudaFree(g.side_buf[p]);
     g.side_buf[p] = nullptr;
+    g.side_refused[p] = false;
     g.side_P[p] = nullptr;
     g.side_up[p] = nullptr;
     g.face_c[p] = nullptr;

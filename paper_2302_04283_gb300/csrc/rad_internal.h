@@ -128,6 +128,7 @@ struct DevGeom {
   // set where the bin is upwind of its side s
   // one allocation per precision holds them
   void *side_buf[2] = {nullptr, nullptr};
+  bool side_refused[2] = {false, false};    // did not fit the device: not tried again for this metric
   void *side_P[2] = {nullptr, nullptr};
   unsigned char *side_up[2] = {nullptr, nullptr};
   // FP64 only, built with it: n^d n_0 of every x1 face [n2][n1+1][n_ap]

@@ -82,7 +82,7 @@ constexpr size_t kSideTableMax = (size_t)4 << 30;
 void ensure_side_table(rad_ctx *ctx, int precision) {
   DevGeom &G = ctx->geom;
   const int ip = precision == RAD_F32 ? 1 : 0;
-  if (G.kind == RAD_MINK_CART || G.side_P[ip]) return;
+  if (G.kind == RAD_MINK_CART || G.side_P[ip] || G.side_refused[ip]) return;
   const size_t ncol = (size_t)G.n[0] * G.n[1], nap = (size_t)ctx->ang.n_ap;
   const size_t nf[2] = {(size_t)G.n[1] * (G.n[0] + 1), (size_t)(G.n[1] + 1) * G.n[0]};
   auto pad = [](size_t b) { return (b + 255) / 256 * 256; };
@@ -103,7 +103,11 @@ void ensure_side_table(rad_ctx *ctx, int precision) {
   unsigned char *buf = nullptr;
   while (cudaMalloc(&buf, bP + bU + bF) != cudaSuccess) {
     cudaGetLastError();
-    if (!bF) return;
+    if (!bF) {
+      // not tried again for this metric: steps after the first allocate nothing
+      G.side_refused[ip] = true;
+      return;
+    }
     bF = 0;
   }
   void *P = buf;

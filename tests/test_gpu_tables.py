@@ -1,4 +1,5 @@
-"""The angular-flux tables of a spherical metric are optional: they are bounded."""
+"""The angular-flux tables of a spherical metric are optional: they are bounded, and a
+table that does not fit the device is left out."""
 import pytest
 import torch
 
@@ -9,6 +10,68 @@ from tests.harness import GpuCase
 pytestmark = pytest.mark.gpu
 
 MIB = 1 << 20
+
+
+def _case(name, n, level, prec, recon_ang, latlong=None):
+    w = W.make(name, n=n, level=level, latlong=latlong)
+    gc = GpuCase(w)
+    tdt = torch.float64 if prec == "f64" else torch.float32
+    I = torch.nn.functional.pad(torch.tensor(w["I0"], dtype=tdt, device="cuda"),
+                                (0, gc.n_ap - gc.n_ang)).contiguous()
+    o = rad.rad_opts_default(precision=rad.RAD_F64 if prec == "f64" else rad.RAD_F32, recon_ang=recon_ang,
+                             coupling=rad.RAD_COUPLE_EMISSIVITY if w["eta"] is not None else
+                             rad.RAD_COUPLE_THERMAL)
+    return w, gc, I, gc.gas(w), rad.rad_cfl_dt(gc.ctx, w["cfl"]), o
+
+
+def _fill(leave):
+    """Hold all device memory but `leave` bytes."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hold = []
+    for _ in range(4):
+        free = torch.cuda.mem_get_info()[0]
+        if free <= leave + 2 * MIB:
+            break
+        hold.append(torch.empty((free - leave) // MIB * MIB, dtype=torch.uint8, device="cuda"))
+    return hold
+
+
+# 256 x 256 columns of 162 bins in FP64: 82 MiB per intensity array, the tables 594 (sides) + 185 (faces) MiB
+BIG = ("adjoint2d", (256, 256, 1), 4, "f64", rad.RAD_RECON_DC)
+
+
+def _load_kernels():
+    """Kernels are loaded on their first use, which takes device memory."""
+    w, gc, I, gas, dt, o = _case("adjoint2d", (8, 8, 1), 4, "f64", rad.RAD_RECON_DC)
+    rad.rad_step(gc.ctx, I, gas, dt, o)
+    gc.close()
+
+
+def test_a_table_that_does_not_fit_is_not_tried_again():
+    """Until the metric is set again, a step after the refusal allocates nothing."""
+    _load_kernels()
+    w, gc, I, gas, dt, o = _case(*BIG)
+    J, K = I.clone(), I.clone()
+    hold = _fill(300 * MIB)
+    try:
+        rad.rad_step(gc.ctx, J, gas, dt, o)
+        rad.rad_check(gc.ctx)
+        hold.clear()
+        torch.cuda.empty_cache()
+        free = torch.cuda.mem_get_info()[0]
+        rad.rad_step(gc.ctx, K, gas, dt, o)
+        assert torch.cuda.mem_get_info()[0] == free
+        assert torch.equal(J, K)
+        rad.rad_set_metric(gc.ctx, w["kind"], w["spin"], w["ndim"], w["xf"], w["bc"])
+        rad.rad_step(gc.ctx, I, gas, dt, o)
+        rad.rad_check(gc.ctx)
+        assert torch.cuda.mem_get_info()[0] < free - 700 * MIB
+        assert torch.equal(I, K)
+    finally:
+        hold.clear()
+        torch.cuda.empty_cache()
+        gc.close()
 
 
 def test_tables_stay_within_their_bound():
