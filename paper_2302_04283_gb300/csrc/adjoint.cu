@@ -439,6 +439,7 @@ int launch_adjoint(rad_ctx *ctx, const void *I_n, const rad_gas *gas, double dt,
     }
     ctx->adj_bytes = need;
   }
+  ensure_side_table(ctx, o->precision);      // after the scratch: the call runs without the table
   unsigned char *p = (unsigned char *)ctx->adj_buf;
   void *I1 = p, *I1s = p + ib, *I2s = p + 2 * ib, *mu = p + 3 * ib, *lamI1 = p + 4 * ib;
   double *T1 = (double *)(p + 5 * ib), *T2 = (double *)(p + 5 * ib + tb);

@@ -542,7 +542,6 @@ int rad_step_adjoint(rad_ctx *ctx, const void *I_n, const rad_gas *gas, double d
   if (!(dt > 0.0)) return fail(ctx, RAD_EINVAL, "dt must be > 0");
   if (ctx->ang.n_ang > rad::kMaxBinsStep)
     return fail(ctx, RAD_EUNSUPPORTED, "rad_step_adjoint supports up to 812 bins (geodesic level 9)");
-  rad::ensure_side_table(ctx, o->precision);
   std::string err;
   st = rad::launch_adjoint(ctx, I_n, gas, dt, o, lam_np1, lam_n, lamT_np1, lamT_n, g_aa, g_as, g_eta, err);
   return st == RAD_OK ? st : fail(ctx, st, err);

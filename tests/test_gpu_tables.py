@@ -1,5 +1,6 @@
-"""The angular-flux tables of a spherical metric are optional: they are bounded, and a
-table that does not fit the device is left out."""
+"""The angular-flux tables of a spherical metric are optional: they are bounded, a
+table that does not fit the device is left out, and a call that fits without
+them is not refused because of them."""
 import pytest
 import torch
 
@@ -37,7 +38,14 @@ def _fill(leave):
     return hold
 
 
-# 256 x 256 columns of 162 bins in FP64: 82 MiB per intensity array, the tables 594 (sides) + 185 (faces) MiB
+def _adjoint(gc, I, gas, dt, o):
+    lam, ln = torch.ones_like(I), torch.empty_like(I)
+    gr = [torch.zeros_like(gas["T"]) for _ in range(3)]
+    return lambda: rad.rad_step_adjoint(gc.ctx, I, gas, dt, o, lam, ln, None, None, *gr), [ln] + gr
+
+
+# 256 x 256 columns of 162 bins in FP64: 82 MiB per intensity array, the adjoint's scratch 416 MiB, the tables
+# 594 (sides) + 185 (faces) MiB
 BIG = ("adjoint2d", (256, 256, 1), 4, "f64", rad.RAD_RECON_DC)
 
 
@@ -45,6 +53,7 @@ def _load_kernels():
     """Kernels are loaded on their first use, which takes device memory."""
     w, gc, I, gas, dt, o = _case("adjoint2d", (8, 8, 1), 4, "f64", rad.RAD_RECON_DC)
     rad.rad_step(gc.ctx, I, gas, dt, o)
+    _adjoint(gc, I, gas, dt, o)[0]()
     gc.close()
 
 
@@ -68,6 +77,21 @@ def test_a_table_that_does_not_fit_is_not_tried_again():
         rad.rad_check(gc.ctx)
         assert torch.cuda.mem_get_info()[0] < free - 700 * MIB
         assert torch.equal(I, K)
+    finally:
+        hold.clear()
+        torch.cuda.empty_cache()
+        gc.close()
+
+
+def test_adjoint_takes_its_scratch_before_the_tables():
+    _load_kernels()
+    w, gc, I, gas, dt, o = _case(*BIG)
+    run, outs = _adjoint(gc, I, gas, dt, o)
+    hold = _fill(840 * MIB)         # the side table and the scratch do not both fit
+    try:
+        run()
+        rad.rad_check(gc.ctx)
+        assert all(torch.isfinite(t).all() for t in outs)
     finally:
         hold.clear()
         torch.cuda.empty_cache()
