@@ -216,6 +216,8 @@ int rad_cfl_dt(rad_ctx *ctx, double cfl, double *dt_out);
  * spherical metric a table of the angular-flux prefactors per precision (7
  * values per column and bin, FP64 also 2 per face; 4 GiB per precision at
  * most, and not while the stream is captured: the same results without it).
+ * A scratch allocation that does not fit beside it takes its place, unless a
+ * step was captured into a graph that reads it.
  * Geodesic levels up to 9 (812 bins: one CTA of at most 512 threads holds
  * every bin of a cell) and fewer than 2^32 intensity elements per block;
  * RAD_EUNSUPPORTED otherwise.

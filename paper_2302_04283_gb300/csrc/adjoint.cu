@@ -87,7 +87,7 @@ int launch_loss(rad_ctx *ctx, const void *I, int precision, double *L, void *dL,
     cudaFree(ctx->loss_buf);
     ctx->loss_buf = nullptr;
     ctx->loss_rows = 0;
-    if (cudaMalloc(&ctx->loss_buf, rows * sizeof(double)) != cudaSuccess) {
+    if (alloc_scratch(ctx, (void **)&ctx->loss_buf, rows * sizeof(double)) != cudaSuccess) {
       err = "loss scratch allocation failed";
       return RAD_ENOMEM;
     }
@@ -433,7 +433,7 @@ int launch_adjoint(rad_ctx *ctx, const void *I_n, const rad_gas *gas, double dt,
     cudaFree(ctx->adj_buf);
     ctx->adj_buf = nullptr;
     ctx->adj_bytes = 0;
-    if (cudaMalloc(&ctx->adj_buf, need) != cudaSuccess) {
+    if (alloc_scratch(ctx, &ctx->adj_buf, need) != cudaSuccess) {
       err = "adjoint scratch allocation failed";
       return RAD_ENOMEM;
     }

@@ -347,6 +347,7 @@ void free_geometry(DevGeom &g) {
     g.face_c[p] = nullptr;
     g.face_up[p] = nullptr;
   }
+  g.side_captured = false;
   g.cols = nullptr;
   g.f1 = g.f2 = g.f3 = nullptr;
   g.colsF = nullptr;

@@ -62,7 +62,7 @@ extern "C" int rad_step_host(rad_ctx *ctx, int n_items, const rad_host_item *ite
     cudaFree(ctx->host_slot_buf);
     ctx->host_slot_buf = nullptr;
     ctx->host_slot_bytes = 0;
-    if (cudaMalloc(&ctx->host_slot_buf, NS * per_slot) != cudaSuccess)
+    if (rad::alloc_scratch(ctx, &ctx->host_slot_buf, NS * per_slot) != cudaSuccess)
       return fail_h(ctx, RAD_ENOMEM, "rad_step_host: slot allocation failed");
     ctx->host_slot_bytes = NS * per_slot;
   }

@@ -378,7 +378,7 @@ static int build_wt(rad_ctx *ctx, int kp, std::string &err) {
   }
   cudaFree(ctx->wt_dev);
   ctx->wt_dev = nullptr;
-  if (cudaMalloc(&ctx->wt_dev, buf.size() * 2) != cudaSuccess) {
+  if (alloc_scratch(ctx, (void **)&ctx->wt_dev, buf.size() * 2) != cudaSuccess) {
     err = "moment weight allocation failed";
     return RAD_ENOMEM;
   }

@@ -129,6 +129,7 @@ struct DevGeom {
   // one allocation per precision holds them
   void *side_buf[2] = {nullptr, nullptr};
   bool side_refused[2] = {false, false};    // did not fit the device: not tried again for this metric
+  bool side_captured = false;               // a captured graph may read them: kept until the metric is set again
   void *side_P[2] = {nullptr, nullptr};
   unsigned char *side_up[2] = {nullptr, nullptr};
   // FP64 only, built with it: n^d n_0 of every x1 face [n2][n1+1][n_ap]
@@ -218,6 +219,12 @@ cudaError_t launch_wait_selftest(rad_ctx *ctx, double seconds);
 // fluxes and the table is worth its memory; without one the kernels compute
 // the prefactors themselves (the same values)
 void ensure_side_table(rad_ctx *ctx, int precision);
+// cudaMalloc for what a call cannot do without: on a full device the tables
+// are given up first (unless a captured graph may read them).  A failure
+// leaves no error behind for later launches.
+cudaError_t alloc_scratch(rad_ctx *ctx, void **p, size_t bytes);
+// before launches that read the tables: are they being captured into a graph?
+void note_capture(rad_ctx *ctx);
 
 // moments.cu
 int launch_moments(rad_ctx *ctx, const void *I, int precision, int frame, int method,

@@ -143,4 +143,34 @@ void ensure_side_table(rad_ctx *ctx, int precision) {
   }
 }
 
+cudaError_t alloc_scratch(rad_ctx *ctx, void **p, size_t bytes) {
+  cudaError_t ce = cudaMalloc(p, bytes);
+  if (ce == cudaSuccess) return ce;
+  cudaGetLastError();                    // handled here: later launches look at this state too
+  DevGeom &G = ctx->geom;
+  if (!(G.side_buf[0] || G.side_buf[1]) || G.side_captured) return ce;
+  cudaStreamSynchronize(ctx->stream);
+  for (int ip = 0; ip < 2; ++ip) {
+    cudaFree(G.side_buf[ip]);
+    G.side_buf[ip] = G.side_P[ip] = nullptr;
+    G.side_up[ip] = nullptr;
+    G.face_c[ip] = nullptr;
+    G.face_up[ip] = nullptr;
+    G.side_refused[ip] = true;
+  }
+  ce = cudaMalloc(p, bytes);
+  if (ce != cudaSuccess) cudaGetLastError();
+  return ce;
+}
+
+void note_capture(rad_ctx *ctx) {
+  DevGeom &G = ctx->geom;
+  if (G.side_captured || !(G.side_buf[0] || G.side_buf[1])) return;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    G.side_captured = true;
+  }
+}
+
 }  // namespace rad

@@ -182,6 +182,7 @@ StageArgs make_stage_args(rad_ctx *ctx, const rad_gas *gas, double dt, const rad
     a.face_c[d] = both ? G.face_c[d] : nullptr;
     a.face_up[d] = both ? G.face_up[d] : nullptr;
   }
+  note_capture(ctx);
   a.side_P = G.side_P[o->precision == RAD_F32];
   a.side_up = G.side_up[o->precision == RAD_F32];
   a.edge_pq = ctx->dang.edge_pq;
@@ -329,7 +330,7 @@ int launch_step(rad_ctx *ctx, void *I, const rad_gas *gas, double dt, const rad_
 int launch_cfl(rad_ctx *ctx, double cfl, double *dt_out, std::string &err) {
   const DevGeom &G = ctx->geom;
   unsigned long long *d = nullptr;
-  if (cudaMalloc(&d, sizeof(unsigned long long)) != cudaSuccess) {
+  if (alloc_scratch(ctx, (void **)&d, sizeof(unsigned long long)) != cudaSuccess) {
     err = "cfl: allocation failed";
     return RAD_ENOMEM;
   }

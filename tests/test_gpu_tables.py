@@ -98,6 +98,55 @@ def test_adjoint_takes_its_scratch_before_the_tables():
         gc.close()
 
 
+def test_tables_make_room_for_a_later_scratch():
+    _load_kernels()
+    w, gc, I, gas, dt, o = _case(*BIG)
+    J, K = I.clone(), I.clone()
+    run, outs = _adjoint(gc, I, gas, dt, o)
+    rad.rad_step(gc.ctx, J, gas, dt, o)          # builds the tables
+    hold = _fill(300 * MIB)                      # less than the adjoint's scratch
+    try:
+        run()
+        rad.rad_step(gc.ctx, K, gas, dt, o)
+        rad.rad_check(gc.ctx)
+        assert torch.equal(J, K)
+    finally:
+        hold.clear()
+        torch.cuda.empty_cache()
+        gc.close()
+
+
+def test_a_captured_step_keeps_its_tables():
+    """Tables that a captured graph reads are not given up: the graph replays
+    after a call that did not fit."""
+    _load_kernels()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        w, gc, I, gas, dt, o = _case(*BIG)
+        J = I.clone()
+        run, outs = _adjoint(gc, I, gas, dt, o)
+        rad.rad_step(gc.ctx, J, gas, dt, o)
+        ref = J.clone()
+        s.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            rad.rad_step(gc.ctx, J, gas, dt, o)
+    hold = _fill(300 * MIB)
+    try:
+        with torch.cuda.stream(s):
+            with pytest.raises(rad.RadError):
+                run()
+            J.copy_(I)
+            graph.replay()
+            s.synchronize()
+            rad.rad_check(gc.ctx)
+            assert torch.equal(J, ref)
+    finally:
+        hold.clear()
+        torch.cuda.empty_cache()
+        gc.close()
+
+
 def test_tables_stay_within_their_bound():
     """Side and face tables and their flags count together: 4 GiB."""
     w = W.make("adjoint2d", n=(338, 338, 1), level=8, with_intensity=False)
