@@ -51,7 +51,7 @@ __global__ void k_side_table(const Col *__restrict__ cols, int nang, int nap, co
 }
 
 // One CTA per face; FP64 prefactors n^d n_0 of the spatial fluxes (the stage
-// kernel's operations, so that it gives the same bits with and without).
+// and adjoint kernels' operations, so that they give the same bits with and without).
 __global__ void k_face_table(const FaceGeo *__restrict__ faces, int nang, int nap, const double *__restrict__ dir,
                              double *__restrict__ c, unsigned char *__restrict__ up) {
   const size_t f = blockIdx.x;
@@ -59,12 +59,7 @@ __global__ void k_face_table(const FaceGeo *__restrict__ faces, int nang, int na
   for (int n = threadIdx.x; n < nap; n += blockDim.x) {
     double v = 0.0;
     bool u = false;
-    if (n < nang) {
-      const double x = dir[3 * n], y = dir[3 * n + 1], z = dir[3 * n + 2];
-      const double na = fma_rn(F.ea[3], z, fma_rn(F.ea[2], y, fma_rn(F.ea[1], x, F.ea[0])));
-      v = mul_rn(na, fma_rn(F.m0[3], z, fma_rn(F.m0[2], y, fma_rn(F.m0[1], x, F.m0[0]))));
-      u = na < 0.0;
-    }
+    if (n < nang) v = face_nd_n0(F, dir[3 * n], dir[3 * n + 1], dir[3 * n + 2], u);
     c[f * nap + n] = v;
     up[f * nap + n] = u;
   }

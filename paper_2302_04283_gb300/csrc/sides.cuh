@@ -35,6 +35,15 @@ __device__ __forceinline__ R side_prefactor(const Col &cg, const double *eg, boo
   return mul_rn(mul_rn(len, sp), n0);
 }
 
+// FP64 prefactor n^d n_0 of a face for a direction, and whether n^d < 0 (the
+// upwind cell is the upper one).
+template <typename Face>
+__device__ __forceinline__ double face_nd_n0(const Face &F, double x, double y, double z, bool &upR) {
+  const double na = fma_rn(F.ea[3], z, fma_rn(F.ea[2], y, fma_rn(F.ea[1], x, F.ea[0])));
+  upR = na < 0.0;
+  return mul_rn(na, fma_rn(F.m0[3], z, fma_rn(F.m0[2], y, fma_rn(F.m0[1], x, F.m0[0]))));
+}
+
 // v per solid angle of bin n: a quotient in FP32, a product with the
 // tabulated reciprocal in FP64 (a division costs ten operations of the FP64
 // pipe).

@@ -1,6 +1,7 @@
-"""The angular-flux tables of a spherical metric are optional: they are bounded, a
-table that does not fit the device is left out, and a call that fits without
-them is not refused because of them."""
+"""The angular-flux tables of a spherical metric are optional: a call gives
+the same bits with and without them, they are bounded, a table that
+does not fit the device is left out, and a call that fits without them is not
+refused because of them."""
 import pytest
 import torch
 
@@ -23,6 +24,62 @@ def _case(name, n, level, prec, recon_ang, latlong=None):
                              coupling=rad.RAD_COUPLE_EMISSIVITY if w["eta"] is not None else
                              rad.RAD_COUPLE_THERMAL)
     return w, gc, I, gc.gas(w), rad.rad_cfl_dt(gc.ctx, w["cfl"]), o
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("name,n,level,recon_ang,latlong", [
+    ("torus3d_big", (9, 7, 8), 2, rad.RAD_RECON_DC, None),       # inner and boundary cells
+    ("adjoint2d", (11, 9, 1), 3, rad.RAD_RECON_DC, None),
+    ("torus3d_big", (6, 6, 4), 1, rad.RAD_RECON_MAPR, None),
+    ("torus3d_big", (6, 6, 4), 2, rad.RAD_RECON_PLM, (3, 6)),
+])
+def test_stages_and_adjoint_without_tables(name, n, level, recon_ang, latlong, prec):
+    """Run once with the tables, then captured into a graph right after the
+    metric is set again: a captured call builds none."""
+    w, gc, I0, gas, dt, o = _case(name, n, level, prec, recon_ang, latlong)
+    try:
+        g = torch.Generator(device="cuda").manual_seed(3)
+        lam = torch.randn(I0.shape, generator=g, dtype=torch.float64, device="cuda").to(I0.dtype)
+        thermal = gas["eta"] is None
+        I, T = I0.clone(), gas["T"].clone()
+        src = torch.zeros(I.shape[:-1] + (4,), dtype=torch.float64, device="cuda")
+        lT = torch.randn(T.shape, generator=g, dtype=torch.float64, device="cuda") if thermal else None
+        ln, lTn = torch.zeros_like(I), torch.zeros_like(T)
+        ga, gs, ge = (torch.zeros_like(T) for _ in range(3))
+        outs = [I, T, src, ln, lTn, ga, gs, ge]
+
+        def calls():
+            I.copy_(I0)
+            T.copy_(gas["T"])
+            for t in outs[2:]:
+                t.zero_()
+            for stage in (1, 2):
+                rad.rad_step_stage(gc.ctx, stage, I, {**gas, "T": T}, dt, o, src)
+            rad.rad_step_adjoint(gc.ctx, I0, gas, dt, o, lam, ln, lT, lTn if thermal else None, ga, gs,
+                                 None if thermal else ge)
+
+        calls()
+        torch.cuda.synchronize()
+        with_tables = [t.clone() for t in outs]
+        # a context on the stream that is captured; its scratch exists before the tables are dropped
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            gc.close()
+            gc = GpuCase(w)
+            calls()
+            rad.rad_set_metric(gc.ctx, w["kind"], w["spin"], w["ndim"], w["xf"], w["bc"])
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=s):
+                calls()
+            for t in outs:
+                t.zero_()
+            graph.replay()
+        s.synchronize()
+        rad.rad_check(gc.ctx)
+        for a, b in zip(outs, with_tables):
+            assert torch.equal(a, b)
+    finally:
+        gc.close()
 
 
 def _fill(leave):
