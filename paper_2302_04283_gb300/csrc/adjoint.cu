@@ -235,6 +235,13 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
   }
   __syncthreads();
   // ---- phase B
+  // what the forward stage reports of a cell (the recomputation of stage 2 stops
+  // before its coupling): no root, or a source term S past the range of FP64
+  // (no convergence) or of the intensities (they come out non-finite)
+  auto report = [&](bool ok, double S) {
+    if (!ok || !isfinite(S)) atomicOr(a.err, kErrNoConv);
+    else if (sizeof(R) == 4 && !isfinite((float)S)) atomicOr(a.err, kErrNonFinite);
+  };
   for (int c = n; c < nc; c += blockDim.x) {
     const size_t cell = (size_t)(k0 + c) * ncol + col;
     W t[4] = {W(0), W(0), W(0), W(0)};
@@ -257,9 +264,9 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
       const double B4 = A2 * aad * ar, B1 = cv * (1.0 - A2 * asd), B0 = D + A2 * asd * Em - B1 * Tm;
       bool ok = true;
       const double Tp = quartic_root(B4, B1, B0, true, ok, Tm);
-      if (!ok || !isfinite(Tp)) atomicOr(a.err, kErrNoConv);
       const double T3 = Tp * Tp * Tp, T4 = T3 * Tp;
       const double Ep = Em - cv * (Tp - Tm);
+      report(ok && isfinite(Tp), aad * ar * T4 + asd * Ep);
       double lT = (A.lamTp ? A.lamTp[cell] : 0.0) + 4.0 * aad * ar * T3 * lS;
       const double lEp = asd * lS;
       double laa = ar * T4 * lS, las = Ep * lS;
@@ -293,6 +300,11 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
       const W Q = W(1) - A2 * as;
       const W Ep = (A1 + W(kFourPi) * A2 * eta) / Q;
       const W S = W(kFourPi) * eta + as * Ep;
+      if (!isfinite(S)) {                   // S as the forward stage forms it, in FP64
+        const double A2d = a.dts / kFourPi * (double)t[1], asd = a.as[cell], etad = a.eta[cell];
+        const double Epd = ((double)A1 + kFourPi * A2d * etad) / (1.0 - A2d * asd);
+        report(true, kFourPi * etad + asd * Epd);
+      }
       const W lEp = as * lS;
       const W lA1 = lEp / Q;
       const W lQ = -Ep * lEp / Q;
