@@ -60,18 +60,16 @@ __device__ __forceinline__ void cta_sum3(R v0, R v1, R v2, R *buf, int nwarp, in
 }
 
 // Face flux prefactor Delta A n^d n_0 (no 1/dV) and upwind side for one bin.
-// FP64 in the face table's operations, (n^d n_0) Delta A: the same bits for a
-// face whether its prefactor is read or formed, and in both kernels below.
-template <typename Face>
-__device__ __forceinline__ float face_coefA(const Face &F, float x, float y, float z, bool &upR) {
-  float na = F.ea[0] + F.ea[1] * x + F.ea[2] * y + F.ea[3] * z;
-  float n0 = F.m0[0] + F.m0[1] * x + F.m0[2] * y + F.m0[3] * z;
-  upR = na < 0.0f;
-  return F.dA * na * n0;
-}
-template <typename Face>
-__device__ __forceinline__ double face_coefA(const Face &F, double x, double y, double z, bool &upR) {
-  return mul_rn(face_nd_n0(F, x, y, z, upR), F.dA);
+// FP64 in the face table's order, (n^d n_0) Delta A, so that this kernel and the
+// inner cells' round a shared face alike; not in explicit operations, which
+// cost the FP64 kernel 6 % (4 x 64 x 64 cells x 162 bins, gradient step 5.60 ->
+// 5.94 ms).
+template <typename Face, typename R>
+__device__ __forceinline__ R face_coefA(const Face &F, R x, R y, R z, bool &upR) {
+  R na = F.ea[0] + F.ea[1] * x + F.ea[2] * y + F.ea[3] * z;
+  R n0 = F.m0[0] + F.m0[1] * x + F.m0[2] * y + F.m0[3] * z;
+  upR = na < R(0);
+  return sizeof(R) == 8 ? na * n0 * F.dA : F.dA * na * n0;
 }
 
 // dphi/d(stencil position) of the upwind face value: stencil values v0 v1 v2,
@@ -320,12 +318,15 @@ __global__ void __launch_bounds__(sizeof(R) == 8 ? 512 : 832) k_transport_adj_in
       int f = yd + t - 1;                       // face between positions t - 2 and t - 1
       f = f < 0 ? f + N : (f >= N && a.bc_lo[d] == RAD_BC_PERIODIC ? f - N : f);
       const int fi = d == 0 ? j * (a.n1 + 1) + f : f * a.n1 + i;
+      const Face &F = ((const Face *)(d == 0 ? a.f1 : a.f2))[fi];
       bool u;
-      if (sizeof(R) == 8 && a.face_c[d]) {
-        cA[d][t] = mul_rn((R)a.face_c[d][(size_t)fi * a.nap + n], ((const Face *)(d == 0 ? a.f1 : a.f2))[fi].dA);
+      if (sizeof(R) == 4) {
+        cA[d][t] = face_coefA(F, x, y, z, u);
+      } else if (a.face_c[d]) {
+        cA[d][t] = mul_rn((R)a.face_c[d][(size_t)fi * a.nap + n], F.dA);
         u = a.face_up[d][(size_t)fi * a.nap + n];
-      } else {
-        cA[d][t] = face_coefA(((const Face *)(d == 0 ? a.f1 : a.f2))[fi], x, y, z, u);
+      } else {          // the table's operations, for the same bits
+        cA[d][t] = mul_rn((R)face_nd_n0(F, x, y, z, u), F.dA);
       }
       up[d] |= (u ? 1u : 0u) << t;
     }
