@@ -904,16 +904,20 @@ cudaError_t launch_transport_adj(const AdjArgs &A0, cudaStream_t st) {
   int nchunk = (A.s.n3 + A.s.kc - 1) / A.s.kc;
   dim3 grid((unsigned)((long long)A.s.n1 * A.s.n2 * nchunk));
   const bool tau = A.s.tau_const > 0.0, ppm = A.s.recon == RAD_RECON_PPM;
-  // inner cells of the plain DC / PLM form first (an FP64 CTA of more than
-  // 512 threads would not hold the kernel's registers: general form)
-  A.split = AR == 0 && !tau && !ppm && threads <= (sizeof(R) == 8 ? 512 : 832);
+  // inner cells of the plain DC / PLM form first, where there are any: every
+  // line of flux has to hold five cells (an FP64 CTA of more than 512 threads
+  // would not hold the kernel's registers: general form)
+  const bool plain = AR == 0 && !tau && !ppm && threads <= (sizeof(R) == 8 ? 512 : 832);
+  A.split = plain && A.s.n1 >= 5 && (A.s.ndim < 2 || A.s.n2 >= 5) && (A.s.ndim < 3 || A.s.n3 >= 5);
   if constexpr (AR == 0) {
     if (A.split) k_transport_adj_in<R, ANG><<<grid, threads, 0, st>>>(A);
   }
-  if (A.split && A.s.kc > 2) {
+  if (plain && A.s.kc > 2) {
     // few CTAs of the general kernel have cells left, and each walks its own
     // serially: two cells per CTA (gradient step of 45 x 38 x 33 x 162 FP32 with
-    // outflow along x1, with the coupling adjoint below 80 operations: 4.78 -> 4.07 ms)
+    // outflow along x1, with the coupling adjoint below 80 operations: 4.78 -> 4.07
+    // ms).  Also where no cell is inner and all are left: 4 x 24 x 24 x 42 FP64 1.56
+    // ms with whole lines, 0.88 with two cells; 4 x 64 x 64 x 162 6.78 and 5.60
     A.s.kc = 2;
     nchunk = (A.s.n3 + 1) / 2;
     grid = dim3((unsigned)((long long)A.s.n1 * A.s.n2 * nchunk));
