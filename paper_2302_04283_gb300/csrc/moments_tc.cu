@@ -115,6 +115,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return r;
 }
 
+template <bool ONE>
 __global__ void __launch_bounds__(kTcThreads, 1) k_moments_tc(const float *__restrict__ I, float *__restrict__ out,
                                                             long long ncell, int nap, int nang, int kp,
                                                             const uint4 *__restrict__ wt, int frame,
@@ -160,7 +161,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_moments_tc(const float *__res
   };
 
   const long long ntile = (ncell + kTcM - 1) / kTcM;
-  const int nk = kp / kTcKC;                                        // chunks per tile
+  const int nk = ONE ? 1 : kp / kTcKC;                              // chunks per tile
   const int mytiles = ntile > blockIdx.x ? (int)((ntile - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
   const int nunit = mytiles * nk;                                   // this CTA's chunks
   const long long row_step = (long long)gridDim.x * kTcM;
@@ -267,7 +268,24 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_moments_tc(const float *__res
   } else {
     // ---- epilogue: lane m of a tile's TMEM columns holds the 16 sums of its cell m
     const int ew = warp & 3;                               // TMEM lanes 32 ew .. + 31 are this warp's
+    auto cell_of = [&](int ti) { return (blockIdx.x + (long long)ti * gridDim.x) * kTcM + ew * 32 + lane; };
+    // ONE chunk per tile (64 bins or fewer): four warps of this role in place of
+    // the previous form's sixteen per SM, each of which did it, are the chain of
+    // the whole kernel, so a tile's velocities travel a tile ahead.  Fluid frame,
+    // previous form -> without -> with: 96^3 cells x 42 bins 63.6 -> 74.3 -> 64.7 us,
+    // 12 bins 59.0 -> 63.6 -> 52.2.  With more chunks there is time, and 92 bins lose
+    // by it (101 -> 109 us).
+    double un[3] = {0.0, 0.0, 0.0};
+    auto fetch = [&](int ti) {
+      const long long cell = cell_of(ti);
+      if (frame != RAD_FRAME_FLUID || ti >= mytiles || cell >= ncell) return;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) un[q] = __ldg(u + 3 * cell + q);
+    };
+    if (ONE) fetch(0);
     for (int ti = 0; ti < mytiles; ++ti) {
+      const float nx = (float)un[0], ny = (float)un[1], nz = (float)un[2];
+      if (ONE) fetch(ti + 1);
       ok = mbar_wait(smem_addr(fullD + (ti & 1)), (uint32_t)(ti >> 1) & 1u);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
@@ -282,7 +300,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_moments_tc(const float *__res
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       if (lane == 0) arrive(emptyD + (ti & 1));
-      const long long cell = (blockIdx.x + (long long)ti * gridDim.x) * kTcM + ew * 32 + lane;
+      const long long cell = cell_of(ti);
       if (cell >= ncell) continue;
       float Rt[10];
 #pragma unroll
@@ -300,7 +318,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_moments_tc(const float *__res
 #pragma unroll
             for (int b = 0; b < 4; ++b) L[a][b] = cg.e[a][b];
         } else {
-          const float ux = (float)u[3 * cell], uy = (float)u[3 * cell + 1], uz = (float)u[3 * cell + 2];
+          const float ux = ONE ? nx : (float)u[3 * cell], uy = ONE ? ny : (float)u[3 * cell + 1],
+                      uz = ONE ? nz : (float)u[3 * cell + 2];
           const float uu[3] = {ux, uy, uz};
           const float u0 = sqrtf(1.0f + ux * ux + uy * uy + uz * uz);
           L[0][0] = u0;
@@ -309,7 +328,16 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_moments_tc(const float *__res
             L[0][a + 1] = -uu[a];
             L[a + 1][0] = -uu[a];
 #pragma unroll
-            for (int b = 0; b < 3; ++b) L[a + 1][b + 1] = uu[a] * uu[b] / (1.0f + u0) + (a == b ? 1.0f : 0.0f);
+            for (int b = 0; b < 3; ++b) {
+              // a zero numerator (gas at rest, or along an axis) would take the
+              // division's slow path (64^3 x 32 bins at rest 30.5 -> 20.9 us, 26.1 in the
+              // previous form); asm: the compiler would undo the select
+              const float w = uu[a] * uu[b];
+              float num = w == 0.0f ? 1.0f : w;
+              asm("" : "+f"(num));
+              const float q = num / (1.0f + u0);
+              L[a + 1][b + 1] = (w == 0.0f ? 0.0f : q) + (a == b ? 1.0f : 0.0f);
+            }
           }
         }
         const float R4[4][4] = {{Rt[0], Rt[1], Rt[2], Rt[3]},
@@ -404,7 +432,8 @@ int launch_moments_bf16x3(rad_ctx *ctx, const float *I, int frame, const double 
   }
   // two operand buffers (hi, lo), two W^T chunks, barriers and TMEM slot
   constexpr size_t smem = 4 * (size_t)kATile + 2 * kBChunk + 128;
-  cudaError_t ce = cudaFuncSetAttribute(k_moments_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const auto kernel = kp == kTcKC ? k_moments_tc<true> : k_moments_tc<false>;
+  cudaError_t ce = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (ce != cudaSuccess) {
     err = std::string("split-bf16 moments: ") + cudaGetErrorString(ce);
     return RAD_ECUDA;
@@ -414,9 +443,9 @@ int launch_moments_bf16x3(rad_ctx *ctx, const float *I, int frame, const double 
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   long long ntile = (ncell + kTcM - 1) / kTcM;
   const long long blocks = std::min<long long>(ntile, nsm);        // one persistent CTA per SM
-  k_moments_tc<<<(unsigned)blocks, kTcThreads, smem, st>>>(I, R, ncell, ctx->ang.n_ap, ctx->ang.n_ang, kp,
-                                                                     (const uint4 *)ctx->wt_dev, frame, G.colsF,
-                                                                     G.n[0] * G.n[1], u, ctx->err_word);
+  kernel<<<(unsigned)blocks, kTcThreads, smem, st>>>(I, R, ncell, ctx->ang.n_ap, ctx->ang.n_ang, kp,
+                                                     (const uint4 *)ctx->wt_dev, frame, G.colsF, G.n[0] * G.n[1], u,
+                                                     ctx->err_word);
   ce = cudaGetLastError();
   if (ce != cudaSuccess) {
     err = std::string("split-bf16 moments launch failed: ") + cudaGetErrorString(ce);
