@@ -181,11 +181,14 @@ int launch_moments(rad_ctx *ctx, const void *I, int precision, int frame, int me
   if (method == RAD_MOM_BF16X3) return launch_moments_bf16x3(ctx, (const float *)I, frame, u, (float *)R, st, err);
   const int wpb = 8;
   unsigned blocks = (unsigned)((ncell + wpb - 1) / wpb);
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (precision == RAD_F32)
     k_moments_simt<float><<<blocks, 32 * wpb, 0, st>>>(
         (const float *)I, (float *)R, ncell, G.n[0] * G.n[1], ctx->ang.n_ap, ctx->ang.n_ang, ctx->dang.dir,
         ctx->dang.dOmega, frame, G.cols, u);
-  else if (ctx->ang.n_ang <= kMomMaxBins) {
+  else if (ctx->ang.n_ang <= kMomMaxBins && (ncell > 8ll * nsm || ctx->ang.n_ang <= (frame == RAD_FRAME_TETRAD ? 100 : 256))) {
     const size_t smem = (size_t)ctx->ang.n_ang * 10 * sizeof(double);
     if (smem > 48 * 1024) {
       const cudaError_t ce = cudaFuncSetAttribute(k_moments_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -195,13 +198,17 @@ int launch_moments(rad_ctx *ctx, const void *I, int precision, int frame, int me
       }
     }
     // two CTAs (sixteen warps) per SM keep the FP64 pipe busy; each builds its
-    // table once
-    const long long groups = (ncell + kMomCells - 1) / kMomCells;
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const unsigned grid = (unsigned)std::min<long long>((groups + wpb - 1) / wpb, (long long)nsm * 2);
-    k_moments_f64<<<grid, 32 * wpb, smem, st>>>((const double *)I, (double *)R, ncell, G.n[0] * G.n[1], ctx->ang.n_ap,
+    // table once.  Fewer cells than fill them: CTAs of fewer warps, so that the
+    // pipes of all SMs share them (fluid frame, one CTA per eight warps -> now, and
+    // k_moments_simt: 12^3 cells x 162 bins 30.7 -> 20.7 us, 44.4; 8^3 x 162 30.7 ->
+    // 22.6, 24.6).  Of cells that k_moments_simt takes in one wave of CTAs and many
+    // bins, the table costs more than it saves: 8^3 x 642 bins 59.0, with fewer warps
+    // 46.9, k_moments_simt 38.3; 362 bins 46.6, 34.9, 32.6; without a frame change
+    // 162 bins 17.9 with fewer warps, 15.9.
+    const long long groups = (ncell + kMomCells - 1) / kMomCells, cta = 2ll * nsm;
+    const int wpc = (int)std::min<long long>(wpb, (groups + cta - 1) / cta);
+    const unsigned grid = (unsigned)std::min<long long>((groups + wpc - 1) / wpc, cta);
+    k_moments_f64<<<grid, 32 * wpc, smem, st>>>((const double *)I, (double *)R, ncell, G.n[0] * G.n[1], ctx->ang.n_ap,
                                                ctx->ang.n_ang, ctx->dang.dir, ctx->dang.dOmega, frame, G.cols, u);
   } else
     k_moments_simt<double><<<blocks, 32 * wpb, 0, st>>>(
