@@ -42,9 +42,10 @@ WORKLOAD = "turb3d"
 # van Leer slopes and their weights, the upwind face state); x3 from the
 # register window, 9; the own cell's gathered term, 2.5; the coupling sums,
 # 21; the implicit update and guard, 16; the gas-source terms, 9; ~85.5 per
-# stage (12 of them, the slopes' and the coupling's quotients, run on the
-# integer pipe)
+# stage.  12 of a stage's, the slopes' and the coupling's quotients, run on the
+# integer pipe: rates against the FP64 pipe's peak count the others
 FLOPS_PER_UPDATE = 171
+FP64_PIPE_FLOPS_PER_UPDATE = FLOPS_PER_UPDATE - 24
 FP64_PEAK_TFLOPS = 1.25
 WORKLOAD_TEXT = ("turb3d: flat-space Cartesian 128^3, geodesic level 4 (162 bins), periodic, moving gas "
                  "|v|<=0.5, log-uniform opacities, PLM, thermal coupling")
@@ -328,11 +329,12 @@ def run_ours(args, rank, world):
     if args.precision == "f64":
         # the FP64 path is bound by the FP64 pipe: rate against GB300's nominal
         # 1.25 TFLOP/s FP64 (FMA = 2 flops, a division counted as 1)
-        tflops = FLOPS_PER_UPDATE * ncell * na * args.steps / (stage_ms * 1e-3) / 1e12
+        tflops = FP64_PIPE_FLOPS_PER_UPDATE * ncell * na * args.steps / (stage_ms * 1e-3) / 1e12
         meas = rad.rad_fp64_fma_rate(3.0)
         roof = {"bound": "alu", "achieved": round(tflops, 4), "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                 "frac": round(tflops / FP64_PEAK_TFLOPS, 4), "traffic": None,
                 "kernel": "k_stage (both stages)", "flops_per_update": FLOPS_PER_UPDATE,
+                "fp64_pipe_flops_per_update": FP64_PIPE_FLOPS_PER_UPDATE,
                 "peak_source": "nominal FP64 rate", "hbm_achieved_gbs": round(achieved, 1),
                 "peak_measured": round(meas, 4), "frac_of_measured": round(tflops / meas, 4),
                 "peak_measured_source": "rad_fp64_fma_rate: DFMA chains on every SM, CUDA events"}
@@ -490,14 +492,15 @@ def run_extras(args, dev):
     gas["T"].copy_(T0)
     ms64 = _time_steps(s64, 3, 1)
     rad.rad_check(ctx)
-    fp64_tf = FLOPS_PER_UPDATE * ncell * na / (ms64 * 1e-3) / 1e12
+    fp64_tf = FP64_PIPE_FLOPS_PER_UPDATE * ncell * na / (ms64 * 1e-3) / 1e12
     fp64_meas = rad.rad_fp64_fma_rate(3.0)
     out["f64_plain"] = {"value": ncell * na / (ms64 * 1e-3), "unit": "cell-angle updates/s", "ms_per_step": ms64,
                         "fp64_tflops": fp64_tf,
                         "fp64_peak_tflops": FP64_PEAK_TFLOPS,
                         "fp64_peak_tflops_measured": round(fp64_meas, 4),
                         "frac_of_measured_fp64": round(fp64_tf / fp64_meas, 4),
-                        "what": "rad_step FP64 + rad_moments FP64 on CUDA cores, same workload, 3 steps; "
+                        "what": "rad_step FP64 + rad_moments FP64 on CUDA cores, same workload, 3 steps; rate of the "
+                                "operations on the FP64 pipe; "
                                 "peak measured live by rad_fp64_fma_rate (DFMA chains on every SM)"}
     rad.rad_destroy(ctx)
     del I64, I32, Rb

@@ -126,8 +126,9 @@ int launch_loss(rad_ctx *ctx, const void *I, int precision, double *L, void *dL,
 // per cell with one active lane, between the barriers of that cell, cost as
 // many of them as the bins themselves; phase B solves a chunk's cells in one
 // warp.  Every quotient comes from one reciprocal of n^0bar den in place of
-// six correctly rounded divisions of about ten FP64 operations each.  45 x 38 x 33 cells x 162 bins, thermal, FP32 intensities: 5.24 ->
-// 1.32 ms per stage; 256 x 128 x 162, fixed emissivity, FP64: 2.69 -> 1.17 ms.
+// six correctly rounded divisions of about ten FP64 operations each.  45 x 38 x
+// 33 cells x 162 bins, thermal, FP32 intensities: 5.24 -> 1.32 ms per stage; 256
+// x 128 x 162, fixed emissivity, FP64: 2.69 -> 1.17 ms.
 // The thermal sweep runs in FP64 in both precisions (only I* and
 // lambda_I+ are in the working precision): the terms of dL/dalpha_s cancel,
 // and FP32 per-bin sums lose percents.

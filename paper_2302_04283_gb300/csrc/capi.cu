@@ -384,7 +384,8 @@ static int ensure_scratch(rad_ctx *ctx, const rad_opts *o) {
     cudaFree(ctx->freq_buf);
     ctx->freq_buf = nullptr;
     ctx->freq_bytes = 0;
-    if (rad::alloc_scratch(ctx, &ctx->freq_buf, need) != cudaSuccess) return fail(ctx, RAD_ENOMEM, "frequency scratch allocation failed");
+    if (rad::alloc_scratch(ctx, &ctx->freq_buf, need) != cudaSuccess)
+      return fail(ctx, RAD_ENOMEM, "frequency scratch allocation failed");
     ctx->freq_bytes = need;
   }
   if (ctx->scratch_I_bytes < need) {
@@ -392,7 +393,8 @@ static int ensure_scratch(rad_ctx *ctx, const rad_opts *o) {
     cudaFree(ctx->scratch_I);
     ctx->scratch_I = nullptr;
     ctx->scratch_I_bytes = 0;
-    if (rad::alloc_scratch(ctx, &ctx->scratch_I, need) != cudaSuccess) return fail(ctx, RAD_ENOMEM, "stage scratch allocation failed");
+    if (rad::alloc_scratch(ctx, &ctx->scratch_I, need) != cudaSuccess)
+      return fail(ctx, RAD_ENOMEM, "stage scratch allocation failed");
     ctx->scratch_I_bytes = need;
   }
   if (ctx->scratch_T_count < ncell) {

@@ -188,7 +188,8 @@ int launch_moments(rad_ctx *ctx, const void *I, int precision, int frame, int me
     k_moments_simt<float><<<blocks, 32 * wpb, 0, st>>>(
         (const float *)I, (float *)R, ncell, G.n[0] * G.n[1], ctx->ang.n_ap, ctx->ang.n_ang, ctx->dang.dir,
         ctx->dang.dOmega, frame, G.cols, u);
-  else if (ctx->ang.n_ang <= kMomMaxBins && (ncell > 8ll * nsm || ctx->ang.n_ang <= (frame == RAD_FRAME_TETRAD ? 100 : 256))) {
+  else if (ctx->ang.n_ang <= kMomMaxBins &&
+           (ncell > 8ll * nsm || ctx->ang.n_ang <= (frame == RAD_FRAME_TETRAD ? 100 : 256))) {
     const size_t smem = (size_t)ctx->ang.n_ang * 10 * sizeof(double);
     if (smem > 48 * 1024) {
       const cudaError_t ce = cudaFuncSetAttribute(k_moments_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

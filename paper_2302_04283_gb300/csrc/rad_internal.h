@@ -203,7 +203,7 @@ int launch_stage_s(rad_ctx *ctx, int stage, void *I, const rad_gas *gas, double 
                    std::string &err);
 // multigroup: the frequency divergence F_{g+1} - F_g of every group of I into D (frequency.cu)
 int launch_freq_div(rad_ctx *ctx, const void *I, void *D, int precision, std::string &err);
-// one RK2 step of every group (step.cu): frequency divergence, then the stage kernel per group
+// one RK2 step of every group (step.cu): per stage the frequency divergence, then one launch for all groups
 int launch_step_groups(rad_ctx *ctx, void *I, const rad_gas *gas, double dt, const rad_opts *opts,
                        double *gas_src, void *scratch_I, double *scratch_T, void *D, std::string &err);
 // rad_gas_update (gas.cu)
@@ -216,8 +216,8 @@ int launch_cfl(rad_ctx *ctx, double cfl, double *dt_out, std::string &err);
 cudaError_t launch_wait_selftest(rad_ctx *ctx, double seconds);
 
 // sides.cu: build the side table of a precision if the metric has angular
-// fluxes and the table is worth its memory; without one the kernels compute
-// the prefactors themselves (the same values)
+// fluxes and the table fits its bound and the device; without one the kernels
+// compute the prefactors themselves (the same bits)
 void ensure_side_table(rad_ctx *ctx, int precision);
 // cudaMalloc for what a call cannot do without: on a full device the tables
 // are given up first (unless a captured graph may read them).  A failure

@@ -1493,9 +1493,10 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
     }
     // U* = U^{s-1} + dt L   (stage 1)   or   U^0/2 + (U^1 + dt L)/2   (stage 2), L = -(divS + divA)
     if (ANG) sx = P::add(sx, divA);
-    if (EXT && a.divF && FL64)
-      sx = P::fma(kD, __ldg((const V *)((LOC ? gdiv_ : (const R *)a.divF) + (unsigned)(k0 + c) * strideK + own)), sx);
-    else if (EXT && a.divF) sx = P::add(sx, __ldg((const V *)((LOC ? gdiv_ : (const R *)a.divF) + (unsigned)(k0 + c) * strideK + own)));
+    if (EXT && a.divF) {
+      const V df = __ldg((const V *)((LOC ? gdiv_ : (const R *)a.divF) + (unsigned)(k0 + c) * strideK + own));
+      sx = FL64 ? P::fma(kD, df, sx) : P::add(sx, df);
+    }
     // FP64: the affine form (fewer FP64-pipe operations); FP32: U* first and
     // I* after the release (the FP32 kernels' register allocation prefers it)
     constexpr bool AFF = sizeof(R) == 8;
@@ -1575,7 +1576,8 @@ __global__ void __launch_bounds__((sizeof(R) == 4 && !ANG && RC != RAD_RECON_PPM
       for (int w = 0; w < nwarp; ++w)
 #pragma unroll
         for (int r = 0; r < kNRedA; ++r) rs[r] += red[(c * nwarp + w) * kNRedC + r];
-      const double D = sizeof(R) == 8 ? -(double)(sgas[8 * c + 5] * rs[0]) : (double)rs[0], A2 = a.dts / kFourPi * (double)rs[1], Em = (double)rs[2];
+      const double D = sizeof(R) == 8 ? -(double)(sgas[8 * c + 5] * rs[0]) : (double)rs[0];
+      const double A2 = a.dts / kFourPi * (double)rs[1], Em = (double)rs[2];
       double S, Tp = Tst;
       bool ok = true;
       if (a.mode == RAD_COUPLE_THERMAL) {
