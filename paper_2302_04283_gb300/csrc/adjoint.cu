@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
   // before its coupling): no root, or a source term S past the range of FP64
   // (no convergence) or of the intensities (they come out non-finite)
   auto report = [&](bool ok, double S) {
-    if (!ok || !isfinite(S)) atomicOr(a.err, kErrNoConv);
+    if (!ok || exp_ones(S)) atomicOr(a.err, kErrNoConv);      // off the FP64 pipe
     else if (sizeof(R) == 4 && !isfinite((float)S)) atomicOr(a.err, kErrNonFinite);
   };
   for (int c = n; c < nc; c += blockDim.x) {
@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
       const W Q = W(1) - A2 * as;
       const W Ep = (A1 + W(kFourPi) * A2 * eta) / Q;
       const W S = W(kFourPi) * eta + as * Ep;
-      if (!isfinite(S)) {                   // S as the forward stage forms it, in FP64
+      if (D64 ? exp_ones((double)S) : !isfinite(S)) {      // S as the forward stage forms it, in FP64
         const double A2d = a.dts / kFourPi * (double)t[1], asd = a.as[cell], etad = a.eta[cell];
         const double Epd = ((double)A1 + kFourPi * A2d * etad) / (1.0 - A2d * asd);
         report(true, kFourPi * etad + asd * Epd);

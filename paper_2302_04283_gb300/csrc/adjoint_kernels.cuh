@@ -72,6 +72,17 @@ __device__ __forceinline__ R face_coefA(const Face &F, R x, R y, R z, bool &upR)
   return sizeof(R) == 8 ? na * n0 * F.dA : F.dA * na * n0;
 }
 
+// The same for the inner cells, which read the face table in FP64 where there is
+// one: in its operations, for the same bits where there is none.
+template <typename Face>
+__device__ __forceinline__ float face_coef_rn(const Face &F, float x, float y, float z, bool &upR) {
+  return face_coefA(F, x, y, z, upR);
+}
+template <typename Face>
+__device__ __forceinline__ double face_coef_rn(const Face &F, double x, double y, double z, bool &upR) {
+  return mul_rn(face_nd_n0(F, x, y, z, upR), F.dA);
+}
+
 // dphi/d(stencil position) of the upwind face value: stencil values v0 v1 v2,
 // phi = v1 +- q(v0, v1, v2) (+ for the left cell, - for the right cell).
 template <typename R>
@@ -318,22 +329,19 @@ __global__ void __launch_bounds__(sizeof(R) == 8 ? 512 : 832) k_transport_adj_in
       int f = yd + t - 1;                       // face between positions t - 2 and t - 1
       f = f < 0 ? f + N : (f >= N && a.bc_lo[d] == RAD_BC_PERIODIC ? f - N : f);
       const int fi = d == 0 ? j * (a.n1 + 1) + f : f * a.n1 + i;
-      const Face &F = ((const Face *)(d == 0 ? a.f1 : a.f2))[fi];
       bool u;
-      if (sizeof(R) == 4) {
-        cA[d][t] = face_coefA(F, x, y, z, u);
-      } else if (a.face_c[d]) {
-        cA[d][t] = mul_rn((R)a.face_c[d][(size_t)fi * a.nap + n], F.dA);
+      if (sizeof(R) == 8 && a.face_c[d]) {
+        cA[d][t] = mul_rn((R)a.face_c[d][(size_t)fi * a.nap + n], ((const Face *)(d == 0 ? a.f1 : a.f2))[fi].dA);
         u = a.face_up[d][(size_t)fi * a.nap + n];
-      } else {          // the table's operations, for the same bits
-        cA[d][t] = mul_rn((R)face_nd_n0(F, x, y, z, u), F.dA);
+      } else {
+        cA[d][t] = face_coef_rn(((const Face *)(d == 0 ? a.f1 : a.f2))[fi], x, y, z, u);
       }
       up[d] |= (u ? 1u : 0u) << t;
     }
   }
   {
     bool u = false;
-    const R c = (act && a.ndim >= 3) ? face_coefA(((const Face *)a.f3)[col], x, y, z, u) : R(0);
+    const R c = (act && a.ndim >= 3) ? face_coef_rn(((const Face *)a.f3)[col], x, y, z, u) : R(0);
 #pragma unroll
     for (int t = 0; t < 4; ++t) cA[2][t] = c;
 #pragma unroll
