@@ -38,9 +38,9 @@ __device__ __forceinline__ uint64_t quot_digits(uint32_t ah, uint32_t al, uint32
   return ((uint64_t)w1 << 21) + (w2 << 2) + ((uint64_t)(w0 << 10) << 32);
 }
 
-// 1 / x; 0 where 1 / x is below the normal range (x above 2^1022), not a number
-// for zero, subnormal, infinite or NaN x (as the refined hardware
-// approximation gives; callers discard it).
+// 1 / x; not a number for zero, subnormal, infinite or NaN x (as the refined
+// hardware approximation gives; callers discard it) and where 1 / x is not normal
+// (x above 2^1022).
 __device__ __forceinline__ double rcp_digits(double x) {
   const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
   const uint32_t e = h & 0x7ff00000u;
@@ -48,11 +48,9 @@ __device__ __forceinline__ double rcp_digits(double x) {
   const uint32_t top = (uint32_t)(q >> 63);             // significand of x is 1
   q = (q + (512u << top)) >> (10u + top);               // 53 bits, rounded
   const uint32_t hi = (uint32_t)(q >> 32) + 0x3ff00000u - e + ((1021u + top) << 20);
-  // 1 / x is normal for exponents 1 .. 2044; for 2045 and 2046 only the power
-  // of two 2^1022 has a normal reciprocal, which is given up too
+  // 1 / x is normal for exponents 1 .. 2044 (and for the power of two 2^1022)
   const bool ok = e - 0x00100000u < 0x7fc00000u;
-  const uint32_t out = e - 0x7fd00000u < 0x00200000u ? 0u : 0x7ff80000u;
-  return __hiloint2double((int)(ok ? hi | (h & 0x80000000u) : out), ok ? (int)(uint32_t)q : 0);
+  return __hiloint2double(ok ? (int)(hi | (h & 0x80000000u)) : 0x7ff80000, (int)(uint32_t)q);
 }
 
 // van Leer's half-slope dl dr / (dl + dr) where dl and dr have one sign, else
