@@ -236,13 +236,9 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
   }
   __syncthreads();
   // ---- phase B
-  // what the forward stage reports of a cell (the recomputation of stage 2 stops
-  // before its coupling): no root, or a source term S past the range of FP64
+  // reports what the forward stage reports of a cell (the recomputation of stage 2
+  // stops before its coupling): no root, or a source term S past the range of FP64
   // (no convergence) or of the intensities (they come out non-finite)
-  auto report = [&](bool ok, double S) {
-    if (!ok || exp_ones(S)) atomicOr(a.err, kErrNoConv);      // off the FP64 pipe
-    else if (sizeof(R) == 4 && !isfinite((float)S)) atomicOr(a.err, kErrNonFinite);
-  };
   for (int c = n; c < nc; c += blockDim.x) {
     const size_t cell = (size_t)(k0 + c) * ncol + col;
     W t[4] = {W(0), W(0), W(0), W(0)};
@@ -267,7 +263,9 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
       const double Tp = quartic_root(B4, B1, B0, true, ok, Tm);
       const double T3 = Tp * Tp * Tp, T4 = T3 * Tp;
       const double Ep = Em - cv * (Tp - Tm);
-      report(ok && isfinite(Tp), aad * ar * T4 + asd * Ep);
+      const double S = aad * ar * T4 + asd * Ep;
+      if (!ok || !isfinite(Tp) || exp_ones(S)) atomicOr(a.err, kErrNoConv);      // S off the FP64 pipe
+      else if (sizeof(R) == 4 && !isfinite((float)S)) atomicOr(a.err, kErrNonFinite);
       double lT = (A.lamTp ? A.lamTp[cell] : 0.0) + 4.0 * aad * ar * T3 * lS;
       const double lEp = asd * lS;
       double laa = ar * T4 * lS, las = Ep * lS;
@@ -288,7 +286,7 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
       lA2 += -cv * asd * lB1 + aad * ar * lB4;
       las -= cv * A2 * lB1;
       laa += A2 * ar * lB4;
-      o[0] = c2p * (aad * ar * T4 + asd * Ep);   // c2pre S
+      o[0] = c2p * S;                        // c2pre S
       o[1] = lB0;                            // lambda_D
       o[2] = lEm;
       o[3] = c2p * lA2;                      // lambda of sum dOmega rden / n^0bar
@@ -301,11 +299,10 @@ __global__ void __launch_bounds__(MAXT) k_couple_adj(AdjArgs A) {
       const W Q = W(1) - A2 * as;
       const W Ep = (A1 + W(kFourPi) * A2 * eta) / Q;
       const W S = W(kFourPi) * eta + as * Ep;
-      if (D64 ? exp_ones((double)S) : !isfinite(S)) {      // S as the forward stage forms it, in FP64
-        const double A2d = a.dts / kFourPi * (double)t[1], asd = a.as[cell], etad = a.eta[cell];
-        const double Epd = ((double)A1 + kFourPi * A2d * etad) / (1.0 - A2d * asd);
-        report(true, kFourPi * etad + asd * Epd);
-      }
+      // (FP32: 1 - A2 alpha_s may round to 0 or below at great depth, which the
+      // forward stage, in FP64 there, does not report)
+      if ((D64 ? exp_ones((double)S) : !isfinite(S)) && Q > W(0))
+        atomicOr(a.err, sizeof(R) == 8 ? kErrNoConv : kErrNonFinite);
       const W lEp = as * lS;
       const W lA1 = lEp / Q;
       const W lQ = -Ep * lEp / Q;
